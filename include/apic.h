@@ -285,7 +285,9 @@ typedef struct {
   int32_t sort_interval;        /* steps between particle sorts in use (0: none) */
   int32_t win_rows;             /* node rows of the push's shared-memory deposit window in use */
   int32_t chunk_group;          /* consecutive particle chunks a push CTA takes at a time */
-  int32_t chunk_items;          /* FP32 push: particles per thread of a chunk (16: 4096 per chunk, 32: 8192) */
+  int32_t chunk_items;          /* FP32 push: particles per thread of a chunk (16: 4096 per chunk, 32: 8192).
+                                   Where neither apic_autotune nor apic_set_schedule has fixed them, both are
+                                   upper limits: a launch with few particles takes smaller chunks and groups */
   int64_t timed_sorts;          /* particle sorts run inside apic_step_timed */
   double sort_ms;               /* CUDA-event time of those sorts, summed */
 } apic_stats_t;

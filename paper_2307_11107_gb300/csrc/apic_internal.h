@@ -299,8 +299,9 @@ void launch_deposit_all(const DevPtrs& d, int max_grid, int max_n2, cudaStream_t
 #endif
 // win_rows, chunk_group, chunk_items: the deposit window's node rows, the
 // chunks a CTA takes per group and the particles per thread of a chunk of the
-// vector push (16 or 32; 0: the defaults, push_window_rows, 4 and 32 when
-// `particles` (the batch's particle slots) give every CTA two dozen chunks)
+// vector push (16 or 32; 0: the defaults, push_window_rows, 32 when
+// `particles` (the batch's particle slots) give every CTA two dozen chunks,
+// else up to 16 and groups of up to 4 by the particles there are, push_tiles)
 template <class Real>
 void launch_push(const DevPtrs& d, int grid, int max_n2, bool chord, int win_rows, int chunk_group, int chunk_items,
                  long long particles, cudaStream_t s);

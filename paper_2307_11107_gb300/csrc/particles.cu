@@ -27,7 +27,9 @@ namespace {
 #include "bulk_copy.cuh"
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kPushItems = 8;    // particles per thread per chunk
+constexpr int kPushItems = 8;    // particles per thread per chunk at most
+constexpr int kPushItemsMin = kF64 ? 1 : 4;  // ... at least (the vector push moves four at a time)
+constexpr int kPushClaims = kF64 ? 6 : 2;   // claims (groups of chunks) per CTA wanted before chunks and groups grow
 constexpr int kFlushChunks = 31;  // chunks (of 2048 particles) between window flushes at most
 // the vector push: particles per thread per chunk, 16 (4096 per chunk) or 32
 // (8192: fewer barriers per particle, coarser load balance); a window is
@@ -230,8 +232,66 @@ __device__ __forceinline__ Cell locate_c(const PushConst& C, Real x1, Real x2) {
   return c;
 }
 
+// A launch's chunks: `items` particles per thread of a chunk and `group`
+// consecutive chunks per claim, then the prefix of the populations' chunk
+// counts (by warp 0; ends at a CTA barrier).  items, group = 0: chosen from
+// the particles there are, the largest that still give every CTA kPushClaims
+// claims.  Large chunks and groups spare barriers, counter atomics and window
+// flushes, but a launch with fewer claims than CTAs leaves SMs idle: with
+// fixed 2048-particle chunks in groups of four, 2e5 FP64 particles ran on 25
+// CTAs (1.25 ms; 0.16 ms now), 8e3 FP32 ones on two (39 us; 17 us), 4.7e5
+// FP32 ones on 29 (114 us; 30 us).  The FP64 push is bound by its SM's FP64
+// pipe, so it wants more claims (2e6 particles: 1.30 ms with two, 1.07 with
+// six); from 7.5e6 FP32 particles on, the chunks are the earlier ones.
+// The deposit and the tallies are integer sums: no result depends on the tiles.
+struct PushTiles {
+  int items, group;
+};
+
+__device__ __forceinline__ PushTiles push_tiles(const DevPtrs& d, int items, int group, int most, long long* pre,
+                                                PushTiles* sh) {
+  if (threadIdx.x < 32) {
+    const int lane = threadIdx.x;
+    if (items == 0 || group == 0) {
+      long long n = 0;
+      for (int p = lane; p < d.n_pop; p += 32) n += d.ps[p].n;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(kFull, n, o);
+      const long long per = n / ((long long)blockDim.x * gridDim.x);  // particles per thread of the launch
+      if (items == 0) {
+        items = most;
+        while (items > kPushItemsMin && per < (long long)kPushClaims * items) items >>= 1;
+      }
+      if (group == 0) {
+        group = 4;
+        while (group > 1 && per < (long long)kPushClaims * items * group) group >>= 1;
+      }
+    }
+    const long long CH = (long long)items * blockDim.x;
+    long long carry = 0;
+    for (int p0 = 0; p0 < d.n_pop; p0 += 32) {
+      const int p = p0 + lane;
+      const long long c = p < d.n_pop ? (d.ps[p].n + CH - 1) / CH : 0;
+      long long x = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const long long up = __shfl_up_sync(kFull, x, o);
+        if (lane >= o) x += up;
+      }
+      if (p < d.n_pop) pre[p] = carry + x - c;
+      carry += __shfl_sync(kFull, x, 31);
+    }
+    if (lane == 0) {
+      pre[d.n_pop] = carry;
+      *sh = PushTiles{items, group};
+    }
+  }
+  __syncthreads();
+  return *sh;
+}
+
 // One full particle update for slot t of the batch (Sec. 2, Eqs. 8-10, 9).
-// The CTA works on chunks of kPushItems x blockDim consecutive slots of one
+// The CTA works on chunks of up to kPushItems x blockDim consecutive slots of one
 // population (sorted by cell, so a chunk covers few grid rows) and deposits
 // into a shared-memory window of win_rows (<= kWinRows) node rows that is flushed to the
 // global accumulator after each chunk.
@@ -246,7 +306,8 @@ constexpr int kPushUnroll = APIC_PUSH_UNROLL;  // items of the chunk loop unroll
 // kChord: some instance absorbs grazing orbits (APIC_CHORD_ABSORB); the
 // instantiation without it carries no trace of the test.
 template <bool kChord>
-__global__ void __launch_bounds__(256, APIC_PUSH_MIN_BLOCKS) k_push(DevPtrs d, int win_n2, int win_rows, int group) {
+__global__ void __launch_bounds__(256, APIC_PUSH_MIN_BLOCKS) k_push(DevPtrs d, int win_n2, int win_rows, int group,
+                                                                     int chunk_items) {
   // dynamic shared memory: the deposit window, then the chunk prefix over the
   // populations and their constants (sized by the batch, so that a small
   // batch leaves more of the SM's memory to L1 for the field gather)
@@ -257,15 +318,10 @@ __global__ void __launch_bounds__(256, APIC_PUSH_MIN_BLOCKS) k_push(DevPtrs d, i
   PushConst* s_pc = (PushConst*)(s_pre + d.n_pop + 1);
   __shared__ int s_row0, s_wpop, s_nsince, s_newrow0, s_flush, s_gi;
   __shared__ unsigned s_rowmask;  // FP32 window: cell rows that received moments in this chunk
-  const long long CH = (long long)kPushItems * blockDim.x;
-  if (threadIdx.x == 0) {
-    long long a = 0;
-    for (int p = 0; p < d.n_pop; ++p) {
-      s_pre[p] = a;
-      a += (d.ps[p].n + CH - 1) / CH;
-    }
-    s_pre[d.n_pop] = a;
-  }
+  __shared__ PushTiles s_tiles;
+  const PushTiles tiles = push_tiles(d, chunk_items, group, kPushItems, s_pre, &s_tiles);
+  const int items = tiles.items, GS = tiles.group;
+  const long long CH = (long long)items * blockDim.x;
   for (int p = threadIdx.x; p < d.n_pop; p += blockDim.x) {
     const Pop& P = d.pop[p];
     const Inst& I = d.inst[P.inst];
@@ -357,8 +413,7 @@ __global__ void __launch_bounds__(256, APIC_PUSH_MIN_BLOCKS) k_push(DevPtrs d, i
   // groups of `group` consecutive chunks, taken in order from a counter that
   // is cleared before each launch: the CTAs balance themselves, and the CTAs
   // at work read neighbouring memory
-  const int nch = (int)total_chunks;  // chunks of 2048 particles: far below 2^31
-  const int GS = group > 0 ? group : 1;
+  const int nch = (int)total_chunks;  // at least 2^8 particles each: below 2^31
   const int ngroups = (nch + GS - 1) / GS;
   if (threadIdx.x == 0) {
     s_wpop = -1;
@@ -448,11 +503,11 @@ __global__ void __launch_bounds__(256, APIC_PUSH_MIN_BLOCKS) k_push(DevPtrs d, i
    };
    fetch(0);
 #pragma unroll kPushUnroll
-   for (int it = 0; it < kPushItems; ++it) {
+   for (int it = 0; it < items; ++it) {
     const int o = it * (int)blockDim.x;
     const bool active = o < nleft;
     const Real x1 = nx1, cx2 = nx2, cvR = nvR, cvZ = nvZ, cvT = nvT;
-    if (it + 1 < kPushItems) fetch(it + 1);
+    if (it + 1 < items) fetch(it + 1);
     bool alive = active && x1 < Real(0);
     int fate = 0;  // 1 absorbed, 2 escaped
     int key = -1, di = 0, dj = 0;
@@ -668,18 +723,13 @@ __global__ void __launch_bounds__(256, APIC_PUSH4_MIN_BLOCKS) k_push4(DevPtrs d,
   PushConst* s_pc = (PushConst*)(s_pre + d.n_pop + 1);
   __shared__ int s_row0, s_wpop, s_nsince, s_newrow0, s_flush, s_gi;
   __shared__ unsigned s_rowmask;
+  __shared__ PushTiles s_tiles;
   constexpr int kPer = 4;                 // particles per thread and item
-  const long long CH = (long long)chunk_items * blockDim.x;  // particles per chunk
-  const int items = chunk_items / kPer;     // items of kPer x blockDim particles
+  const PushTiles tiles = push_tiles(d, chunk_items, group, 16, s_pre, &s_tiles);
+  const int GS = tiles.group;
+  const long long CH = (long long)tiles.items * blockDim.x;  // particles per chunk
+  const int items = tiles.items / kPer;     // items of kPer x blockDim particles
   const int flush_chunks = (int)(65535 / CH);  // chunks between window flushes at most
-  if (threadIdx.x == 0) {
-    long long a = 0;
-    for (int p = 0; p < d.n_pop; ++p) {
-      s_pre[p] = a;
-      a += (d.ps[p].n + CH - 1) / CH;
-    }
-    s_pre[d.n_pop] = a;
-  }
   for (int p = threadIdx.x; p < d.n_pop; p += blockDim.x) {
     const Pop& P = d.pop[p];
     const Inst& I = d.inst[P.inst];
@@ -749,7 +799,6 @@ __global__ void __launch_bounds__(256, APIC_PUSH4_MIN_BLOCKS) k_push4(DevPtrs d,
     __syncthreads();
   };
   const int nch = (int)total_chunks;
-  const int GS = group > 0 ? group : 1;
   const int ngroups = (nch + GS - 1) / GS;
   if (threadIdx.x == 0) {
     s_wpop = -1;
@@ -1766,10 +1815,10 @@ void launch_push<Real>(const DevPtrs& d, int grid, int max_n2, bool chord, int w
   const void* kern = v4 ? (chord ? (const void*)k_push4<true> : (const void*)k_push4<false>)
                         : (chord ? (const void*)k_push<true> : (const void*)k_push<false>);
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  static int group_env = -1;  // chunks per group (APIC_PUSH_GROUP, default 4: the fastest of 1, 2, 4, 8 measured)
+  static int group_env = -1;  // chunks per group (APIC_PUSH_GROUP)
   if (group_env < 0) {
     const char* e = std::getenv("APIC_PUSH_GROUP");
-    group_env = e ? std::max(1, std::atoi(e)) : 4;
+    group_env = e ? std::max(1, std::atoi(e)) : 0;
   }
   const int group = chunk_group > 0 ? chunk_group : group_env;
   cudaMemsetAsync(d.cnt + 1, 0, sizeof(long long), s);  // the group counter
@@ -1777,13 +1826,13 @@ void launch_push<Real>(const DevPtrs& d, int grid, int max_n2, bool chord, int w
     grid = std::max(1, grid / 4 * (int)APIC_PUSH4_MIN_BLOCKS);  // the caller's grid is 4 CTAs per SM
     // 8192-particle chunks when every CTA still gets two dozen of them
     int ci = chunk_items == 16 || chunk_items == 32 ? chunk_items
-                                                    : (particles >= 24ll * 8192 * grid ? kPush4ItemsMax : 16);
+                                                    : (particles >= 24ll * 8192 * grid ? kPush4ItemsMax : 0);
     if (chord) k_push4<true><<<grid, 256, sm, s>>>(d, win_n2, rows, group, ci);
     else k_push4<false><<<grid, 256, sm, s>>>(d, win_n2, rows, group, ci);
-  } else if (chord) {
-    k_push<true><<<grid, 256, sm, s>>>(d, win_n2, rows, group);
   } else {
-    k_push<false><<<grid, 256, sm, s>>>(d, win_n2, rows, group);
+    grid = std::max(1, grid / 4 * (int)APIC_PUSH_MIN_BLOCKS);
+    if (chord) k_push<true><<<grid, 256, sm, s>>>(d, win_n2, rows, group, 0);
+    else k_push<false><<<grid, 256, sm, s>>>(d, win_n2, rows, group, 0);
   }
 }
 
