@@ -134,7 +134,17 @@ __device__ void absorb_tally(const DevPtrs& d, const Inst& I, const Pop& P, Real
     Real mid = Real(0.5) * (lo + hi);
     Real px = R + vx * tau * mid, py = vy * tau * mid, pz = Z + vz * tau * mid;
     Real rr = sqrt(px * px + py * py + pz * pz);
-    if (rr < r_grain(al, pz / rr)) hi = mid; else lo = mid;
+    bool in;
+    if (kF64) {
+      // r < (1 + sqrt(1 + 4 alpha z / r)) / 2 on squares, times r: no second
+      // root and no division (a warp with one absorbed particle waits for
+      // forty of these on the FP64 pipe)
+      const Real tr = Real(2) * rr - Real(1);
+      in = tr < Real(0) || tr * tr * rr < rr + Real(4) * al * pz;
+    } else {
+      in = rr < r_grain(al, pz / rr);
+    }
+    if (in) hi = mid; else lo = mid;
   }
   Real sm = Real(0.5) * (lo + hi);
   Real px = R + vx * tau * sm, py = vy * tau * sm, pz = Z + vz * tau * sm;

@@ -217,19 +217,40 @@ struct PushConst {
   long long node_off, acc_off;
 };
 
-__device__ __forceinline__ Cell locate_c(const PushConst& C, Real x1, Real x2) {
-  Real u1 = (x1 + Real(1)) / C.h1;
-  Real u2 = (x2 + Real(1)) / C.h2;
-  Cell c;
-  c.i = (int)floor(u1);
-  c.j = (int)floor(u2);
-  c.i = c.i < 0 ? 0 : (c.i > C.n1 - 1 ? C.n1 - 1 : c.i);
-  c.j = c.j < 0 ? 0 : (c.j > C.n2 - 1 ? C.n2 - 1 : c.j);
-  c.f1 = u1 - (Real)c.i;
-  c.f2 = u2 - (Real)c.j;
-  c.f1 = c.f1 < Real(0) ? Real(0) : (c.f1 > Real(1) ? Real(1) : c.f1);
-  c.f2 = c.f2 < Real(0) ? Real(0) : (c.f2 > Real(1) ? Real(1) : c.f2);
+// FP64 cell of a logical coordinate u (in cells) and the fraction in it; a
+// coordinate outside [0, n] takes the edge cell and its edge (the clamps of
+// locate, on the index: FP64 comparisons share the FP64 pipe).
+__device__ __forceinline__ int cell_of(double u, int n, double& f) {
+  const int i = __double2int_rd(u);
+  const int c = min(max(i, 0), n - 1);
+  f = i < 0 ? 0.0 : (i > n - 1 ? 1.0 : u - (double)c);
   return c;
+}
+
+// The same with the fraction in units of 2^-kCellBits (u < 2^12 cells, so the
+// index and the fraction fit a signed 64-bit word; the fraction's rounding is
+// below the resolution of an FP64 coordinate in cells from u = 8 on and below
+// the deposit's own rounding before).
+constexpr int kCellBits = 50;
+__device__ __forceinline__ int cell_fixed(double u, int n, unsigned long long& f) {
+  const long long t = __double2ll_rn(u * (double)(1ll << kCellBits));
+  const int i = (int)(t >> kCellBits);
+  f = i < 0 ? 0ull : (i > n - 1 ? 1ull << kCellBits : (unsigned long long)t & ((1ull << kCellBits) - 1ull));
+  return min(max(i, 0), n - 1);
+}
+
+// Corner weights of the fractions f1, f2 (units of 2^-kCellBits), each the
+// exact product rounded to F bits.
+__device__ __forceinline__ W4 weights_fixed(unsigned long long f1, unsigned long long f2, int F) {
+  const unsigned long long one = 1ull << kCellBits, g1 = one - f1, g2 = one - f2;
+  const int sh = 2 * kCellBits - F;  // F <= 61
+  const unsigned __int128 half = (unsigned __int128)1 << (sh - 1);
+  W4 w;
+  w.w00 = (unsigned long long)(((unsigned __int128)g1 * g2 + half) >> sh);
+  w.w10 = (unsigned long long)(((unsigned __int128)f1 * g2 + half) >> sh);
+  w.w01 = (unsigned long long)(((unsigned __int128)g1 * f2 + half) >> sh);
+  w.w11 = (unsigned long long)(((unsigned __int128)f1 * f2 + half) >> sh);
+  return w;
 }
 
 // A launch's chunks: `items` particles per thread of a chunk and `group`
@@ -593,45 +614,56 @@ __global__ void __launch_bounds__(256, APIC_PUSH_MIN_BLOCKS) k_push(DevPtrs d, i
         }
       }
     } else if (alive) {
-      Real x2 = cx2, vR = cvR, vZ = cvZ, vT = cvT;
-      const Real al = C.al, dt = C.dt;
-      Real r = radius(al, x1, x2);
-      Real sn = sqrt((Real(1) - x2) * (Real(1) + x2));
-      Real R = r * sn, Z = r * x2;
+      // FP64.  The SM's FP64 pipe bounds this path (two lanes per cycle), so
+      // the operations are counted: every division by a root is a product
+      // with a reciprocal or a reciprocal root (two of each instead of
+      // fourteen divisions and five roots), products and sums are fused, cell
+      // indices and deposit weights are integer arithmetic (about 140 FP64
+      // instructions per particle instead of 330: 2e6 particles 1.07 -> 0.50 ms).
+      double x2 = cx2, vR = cvR, vZ = cvZ, vT = cvT;
+      const double al = C.al, dt = C.dt;
+      // Eq. 3: t = 1 + sqrt(1 - 4 alpha x1 x2), r = -t / (2 x1), 1/r = -2 x1 / t
+      const double t = 1.0 + sqrt(fma(-4.0 * al * x1, x2, 1.0));
+      const double y = 1.0 / (x1 * t);
+      const double ir = -2.0 * x1 * x1 * y, r = -0.5 * t * t * y;
+      const double s2 = (1.0 - x2) * (1.0 + x2), sn = sqrt(s2);
+      const double R = r * sn, Z = r * x2;
       // gather (Eq. 10): bilinear node gradients, analytic metric at the particle
-      Cell c = locate_c(C, x1, x2);
-      const int n00 = c.i * C.N2 + c.j;
-      Real2 a00 = Gi[n00], a10 = Gi[n00 + C.N2], a01 = Gi[n00 + 1], a11 = Gi[n00 + C.N2 + 1];
-      Real w00 = (Real(1) - c.f1) * (Real(1) - c.f2), w10 = c.f1 * (Real(1) - c.f2);
-      Real w01 = (Real(1) - c.f1) * c.f2, w11 = c.f1 * c.f2;
-      Real g1 = w00 * a00.x + w10 * a10.x + w01 * a01.x + w11 * a11.x;
-      Real g2 = w00 * a00.y + w10 * a10.y + w01 * a01.y + w11 * a11.y;
-      Metric<Real> m = metric(al, r, x2);
-      Real ER = -(m.x1R * g1 + m.x2R * g2);
-      Real EZ = -(m.x1Z * g1 + m.x2Z * g2);
+      double f1, f2;
+      const int ci = cell_of((x1 + 1.0) * C.ih1, C.n1, f1), cj = cell_of((x2 + 1.0) * C.ih2, C.n2, f2);
+      const int n00 = ci * C.N2 + cj;
+      const Real2 a00 = Gi[n00], a10 = Gi[n00 + C.N2], a01 = Gi[n00 + 1], a11 = Gi[n00 + C.N2 + 1];
+      const double gx0 = fma(f1, a10.x - a00.x, a00.x), gx1 = fma(f1, a11.x - a01.x, a01.x);
+      const double gy0 = fma(f1, a10.y - a00.y, a00.y), gy1 = fma(f1, a11.y - a01.y, a01.y);
+      const double g1 = fma(f2, gx1 - gx0, gx0), g2 = fma(f2, gy1 - gy0, gy0);
+      // dx1/dR = sin (r + 3 alpha x2) / r^3, dx1/dZ = (r x2 + alpha (3 x2^2 - 1)) / r^3
+      // (3 x2^2 - 1 = 2 - 3 sin^2), dx2/dR = -x2 sin / r, dx2/dZ = sin^2 / r
+      const double ar = al * ir, ir2 = ir * ir, sr_ = sn * ir;
+      const double x1R = sn * ir2 * fma(3.0 * ar, x2, 1.0), x1Z = ir2 * fma(ar, fma(-3.0, s2, 2.0), x2);
+      const double ER = fma(x2 * sr_, g2, -x1R * g1), EZ = -fma(x1Z, g1, s2 * ir * g2);
       // Boris in the local frame (R-hat, Theta-hat, Z-hat); Eq. 9's Lorentz
       // terms are those of the field vector -B z-hat.
-      Real h = C.h;
-      Real vx = vR + h * ER, vy = vT, vz = vZ + h * EZ;
-      Real tz = h * (-C.B);
-      Real sz = Real(2) * tz / (Real(1) + tz * tz);
-      Real px_ = vx + vy * tz, py_ = vy - vx * tz;
-      vx = vx + py_ * sz;
-      vy = vy - px_ * sz;
-      vx = vx + h * ER;
-      vz = vz + h * EZ;
+      const double h = C.h, tz = C.tz, sz = C.sz;
+      double vx = fma(h, ER, vR), vy = vT, vz = fma(h, EZ, vZ);
+      const double px_ = fma(vy, tz, vx), py_ = fma(-vx, tz, vy);
+      vx = fma(h, ER, fma(py_, sz, vx));
+      vy = fma(-px_, sz, vy);
+      vz = fma(h, EZ, vz);
       // straight chord, rotation back to the meridional half plane
-      Real Xc = R + vx * dt, Yc = vy * dt, Zn = Z + vz * dt;
-      Real Rn = sqrt(Xc * Xc + Yc * Yc);
-      Real cr = Real(1), sr = Real(0);
-      if (Rn > Real(0)) {
-        cr = Xc / Rn;
-        sr = Yc / Rn;
+      const double Xc = fma(vx, dt, R), Yc = vy * dt, Zn = fma(vz, dt, Z);
+      const double Rn2 = fma(Xc, Xc, Yc * Yc);
+      double cr = 1.0, sr = 0.0;
+      if (Rn2 > 0.0) {
+        const double iR = rsqrt(Rn2);
+        cr = Xc * iR;
+        sr = Yc * iR;
       }
-      Real vRn = cr * vx + sr * vy, vTn = -sr * vx + cr * vy;
-      Real rn = sqrt(Rn * Rn + Zn * Zn);
-      Real x2n = Zn / rn;
-      bool hit = rn < r_grain(al, x2n);
+      const double vRn = fma(cr, vx, sr * vy), vTn = fma(cr, vy, -sr * vx);
+      const double rn2 = fma(Zn, Zn, Rn2), irn = rsqrt(rn2), rn = rn2 * irn;
+      const double x2n = Zn * irn;
+      // inside the grain: r < (1 + sqrt(1 + 4 alpha x2)) / 2, on squares
+      const double tr = fma(2.0, rn, -1.0), gr = fma(4.0 * al, x2n, 1.0);
+      bool hit = tr < 0.0 || tr * tr < gr;
       Real tau = dt;  // chord time up to a point inside the grain
       if (kChord && !hit && (d.inst[d.pop[pop].inst].flags & APIC_CHORD_ABSORB)) {
         const Real se = chord_entry(al, R, Z, vx * dt, vy * dt, vz * dt);
@@ -646,7 +678,7 @@ __global__ void __launch_bounds__(256, APIC_PUSH_MIN_BLOCKS) k_push(DevPtrs d, i
         X1[t0 + o] = Real(2);
         fate = 1;
       } else {
-        Real x1n = x1_at(al, rn, x2n);
+        const double x1n = -irn * fma(al * x2n, irn, 1.0);  // Eq. 2
         if (x1n > C.x1_out) {
           X1[t0 + o] = Real(2);
           fate = 2;
@@ -656,11 +688,11 @@ __global__ void __launch_bounds__(256, APIC_PUSH_MIN_BLOCKS) k_push(DevPtrs d, i
           VR[t0 + o] = vRn;
           VZ[t0 + o] = vz;
           VT[t0 + o] = vTn;
-          Cell cn = locate_c(C, x1n, x2n);
-          key = cn.i * C.N2 + cn.j;
-          di = cn.i;
-          dj = cn.j;
-          w = weights(cn, C.fbits);
+          unsigned long long e1, e2;
+          di = cell_fixed((x1n + 1.0) * C.ih1, C.n1, e1);
+          dj = cell_fixed((x2n + 1.0) * C.ih2, C.n2, e2);
+          key = di * C.N2 + dj;
+          w = weights_fixed(e1, e2, C.fbits);
         }
       }
     }
@@ -1839,11 +1871,16 @@ void launch_push<Real>(const DevPtrs& d, int grid, int max_n2, bool chord, int w
 template <>
 void launch_inject<Real>(const DevPtrs& d, long long max_inj, cudaStream_t s) {
   if (max_inj <= 0) return;
-  // few CTAs, several injections per thread: fewer window flushes
-  unsigned gx = blocks_for(max_inj, 256);
-  gx = gx < 160 ? gx : 160;
+  // FP32: few CTAs, several injections per thread (fewer window flushes).
+  // FP64: a draw is about a thousand FP64 instructions, which two lanes per
+  // cycle and SM work off, so small CTAs spread the draws over every SM
+  // (1200 draws: 37 us on five CTAs of 256 threads)
+  const int threads = kF64 ? 32 : 256;
+  const unsigned most = kF64 ? 608 : 160;
+  unsigned gx = blocks_for(max_inj, threads);
+  gx = gx < most ? gx : most;
   dim3 g(gx, d.n_pop);
-  k_inject<<<g, 256, 0, s>>>(d);
+  k_inject<<<g, threads, 0, s>>>(d);
 }
 
 // Resident CTAs per SM of the two sort passes for grids of up to `rows` cell
