@@ -25,6 +25,7 @@ namespace {
 
 #include "particle_common.cuh"
 #include "bulk_copy.cuh"
+#include "cell_fixed.cuh"
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kPushItems = 8;    // particles per thread per chunk at most
@@ -40,10 +41,6 @@ constexpr int kPushWinRows = 16; // node rows of the push's shared-memory deposi
 constexpr int kWinMaxN2 = 513;   // widest grid row the window holds (larger grids deposit globally)
 constexpr int kInjRows = 3;      // node rows of the injection window (the last two cell rows)
 constexpr int kInjMaxN2 = 512;   // widest grid (cells in x2) the injection window holds
-
-struct W4 {
-  unsigned long long w00, w10, w01, w11;
-};
 
 // Fixed-point cloud-in-cell weights.  FP64: each weight rounded to F bits.
 // FP32: fractions quantised to F/2 bits, weights as exact integer products
@@ -225,32 +222,6 @@ __device__ __forceinline__ int cell_of(double u, int n, double& f) {
   const int c = min(max(i, 0), n - 1);
   f = i < 0 ? 0.0 : (i > n - 1 ? 1.0 : u - (double)c);
   return c;
-}
-
-// The same with the fraction in units of 2^-kCellBits (u < 2^12 cells, so the
-// index and the fraction fit a signed 64-bit word; the fraction's rounding is
-// below the resolution of an FP64 coordinate in cells from u = 8 on and below
-// the deposit's own rounding before).
-constexpr int kCellBits = 50;
-__device__ __forceinline__ int cell_fixed(double u, int n, unsigned long long& f) {
-  const long long t = __double2ll_rn(u * (double)(1ll << kCellBits));
-  const int i = (int)(t >> kCellBits);
-  f = i < 0 ? 0ull : (i > n - 1 ? 1ull << kCellBits : (unsigned long long)t & ((1ull << kCellBits) - 1ull));
-  return min(max(i, 0), n - 1);
-}
-
-// Corner weights of the fractions f1, f2 (units of 2^-kCellBits), each the
-// exact product rounded to F bits.
-__device__ __forceinline__ W4 weights_fixed(unsigned long long f1, unsigned long long f2, int F) {
-  const unsigned long long one = 1ull << kCellBits, g1 = one - f1, g2 = one - f2;
-  const int sh = 2 * kCellBits - F;  // F <= 61
-  const unsigned __int128 half = (unsigned __int128)1 << (sh - 1);
-  W4 w;
-  w.w00 = (unsigned long long)(((unsigned __int128)g1 * g2 + half) >> sh);
-  w.w10 = (unsigned long long)(((unsigned __int128)f1 * g2 + half) >> sh);
-  w.w01 = (unsigned long long)(((unsigned __int128)g1 * f2 + half) >> sh);
-  w.w11 = (unsigned long long)(((unsigned __int128)f1 * f2 + half) >> sh);
-  return w;
 }
 
 // A launch's chunks: `items` particles per thread of a chunk and `group`
@@ -689,10 +660,10 @@ __global__ void __launch_bounds__(256, APIC_PUSH_MIN_BLOCKS) k_push(DevPtrs d, i
           VZ[t0 + o] = vz;
           VT[t0 + o] = vTn;
           unsigned long long e1, e2;
-          di = cell_fixed((x1n + 1.0) * C.ih1, C.n1, e1);
-          dj = cell_fixed((x2n + 1.0) * C.ih2, C.n2, e2);
+          di = cell_fixed(x1n, C.ih1 * kCellOne, C.n1, kCellBits, e1);
+          dj = cell_fixed(x2n, C.ih2 * kCellOne, C.n2, kCellBits, e2);
           key = di * C.N2 + dj;
-          w = weights_fixed(e1, e2, C.fbits);
+          w = weights_fixed(e1, e2, kCellBits, C.fbits);
         }
       }
     }
