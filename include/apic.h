@@ -61,7 +61,7 @@ extern "C" {
 #define APIC_ERR_CUDA (-7)         /* CUDA runtime or allocation failure */
 
 /* precision of the particle arrays and of the Poisson preconditioner */
-#define APIC_FP64 0          /* FP64 particles, FP64 multigrid (parity path) */
+#define APIC_FP64 0          /* FP64 particles, FP64 direct solve or FP64 multigrid (parity path) */
 #define APIC_FP32_REFINED 1  /* FP32 particles; FP32 block cyclic reduction (or FP32 multigrid) inside an
                                 FP64 residual loop */
 
@@ -293,16 +293,19 @@ typedef struct {
 } apic_stats_t;
 
 /* Poisson solvers (chosen at creation) */
-#define APIC_SOLVER_MG_KERNELS 0 /* BiCGSTAB + multigrid V-cycle, one kernel per phase (FP64 batches) */
-#define APIC_SOLVER_MG_COOP 1    /* the same in one cooperative launch per solve (FP64, one instance) */
+#define APIC_SOLVER_MG_KERNELS 0 /* BiCGSTAB + multigrid V-cycle, one kernel per phase (batches) */
+#define APIC_SOLVER_MG_COOP 1    /* the same in one cooperative launch per solve (one instance) */
 #define APIC_SOLVER_BCR 2        /* FP64 iterative refinement around an FP32 block cyclic reduction of
                                     every instance in one cooperative launch (FP32 particles, any n1,
-                                    grids up to 543 cells in x2): the default when the whole batch's
-                                    reduction blocks fit in L2 (e.g. one 256 x 128 grid) */
+                                    grids up to 543 cells in x2): the default for small grids (fewer than
+                                    16384 nodes, up to 96 cells in x2) whose reduction blocks fit in L2 */
 #define APIC_SOLVER_ND 3         /* the same refinement around an FP32 nested-dissection factorisation (formed
                                     once at creation on the host in FP64) for some or all instances: the
                                     default otherwise (larger grids, batches); APIC_DIRECT=bcr / nd / wide
                                     (nested dissection only for grids wider than 256 cells) override */
+#define APIC_SOLVER_ND64 4       /* FP64 particles: the refinement around an FP64 nested-dissection factorisation
+                                    (one pass reaches FP64 rounding), the default; APIC_PRECOND=mg keeps
+                                    multigrid */
 
 /* Counters of the batch (launch counts, Krylov iterations, phase times). */
 int apic_stats(apic_sim* sim, apic_stats_t* out);

@@ -6,12 +6,14 @@ Translation units (compiled in parallel):
   fields.cu     node fields and bookkeeping, the isolated grain's correction and
                 the Newton linearisation of Boltzmann electrons (FP64, -fmad=false)
   bcr.cu        block cyclic reduction solve (FP32 blocks, FP64 refinement)
+  nd_solve.cu   nested-dissection solve as dataflow sweeps (FP32 or FP64 fronts, FP64 refinement)
   apic.cu       host set-up and the C ABI
   tangent.cu    twice: the sensitivity window's particle kernels in FP64
                 (-fmad=false, with its node kernels) and FP32
   deposit_static.cu  the deposit entry point that uses no caller-side allocation
   probe.cu      the FP32 fused-multiply-add throughput probe (the ALU ceiling)
   nd_factor.cpp the host nested-dissection factorisation of the Poisson system
+  nd_records.cpp  its task records for the dataflow sweeps
   adjoint.cu    twice: the reverse sweep of the sensitivity window in FP64 (-fmad=false,
                 with its node kernels) and FP32
 """
@@ -36,12 +38,14 @@ UNITS = [
     ("poisson.cu", "poisson_f32.o", ["-DAPIC_POISSON_REAL=float", "-DAPIC_POISSON_COMMON=0"]),
     ("fields.cu", "fields.o", ["-fmad=false"]),
     ("bcr.cu", "bcr.o", []),
+    ("nd_solve.cu", "nd_solve.o", []),
     ("apic.cu", "apic.o", []),
     ("tangent.cu", "tangent_f64.o", ["-DAPIC_REAL=double", "-DAPIC_TANGENT_COMMON", "-fmad=false"]),
     ("tangent.cu", "tangent_f32.o", ["-DAPIC_REAL=float"]),
     ("deposit_static.cu", "deposit_static.o", ["-fmad=false"]),
     ("probe.cu", "probe.o", []),
     ("nd_factor.cpp", "nd_factor.o", []),
+    ("nd_records.cpp", "nd_records.o", []),
     ("adjoint.cu", "adjoint_f64.o", ["-DAPIC_REAL=double", "-DAPIC_ADJOINT_COMMON", "-fmad=false"]),
     ("adjoint.cu", "adjoint_f32.o", ["-DAPIC_REAL=float"]),
 ]

@@ -17,6 +17,7 @@
 #include "apic_internal.h"
 #include "dual.cuh"
 #include "geom.cuh"
+#include "nd_records.h"
 
 using namespace apic;
 
@@ -965,7 +966,7 @@ static int setup(apic_sim* S) {
   // instance with a field, N2 <= kBcrMaxNWide, the blocks of the batch within the
   // memory budget (APIC_PRECOND=mg keeps multigrid).
   std::vector<BcrInst> bcr_in;
-  std::vector<int32_t> bcr_kind, bcr_pre, bcr_npre, bcr_tpre;
+  std::vector<int32_t> bcr_kind, bcr_pre, bcr_npre;
   long long bcr_rows = 0;  // floats of bcr_f (and of bcr_e)
   int bcr_nb = 0;          // CTAs of the reduction solve
   // nested dissection per instance (APIC_DIRECT=nd: every instance, bcr:
@@ -974,25 +975,32 @@ static int setup(apic_sim* S) {
   std::vector<NdFactor> nds(ni);
   std::vector<char> use_nd(ni, 0);
   NdUpload ndu;
-  std::vector<int2> nd_flow;      // the dataflow sweeps' task orders
-  std::vector<int32_t> nd_need;   // tasks per front and sweep
-  long long nd_w = 0;  // floats of one right-hand side's update vectors
+  std::vector<NdFlowTask> nd_tasks;   // the dataflow sweeps' records ...
+  std::vector<int64_t> nd_off;        // ... and their first words (of all instances' records)
+  std::vector<int32_t> nd_place, nd_perm;  // a front's first place among its instance's unknowns, an unknown's place
+  std::vector<int4> nd_list;          // the sweeps' record lists
+  long long nd_w = 0;  // elements of one right-hand side's update vectors
+  constexpr int kElem = (int)(sizeof(Real) / sizeof(float));  // words per element of a dataflow solve's fronts
   {
     const char* pc = std::getenv("APIC_PRECOND");
-    bool want = sizeof(Real) == 4 && ni <= kCoopMaxInst && !(pc && std::string(pc) == "mg");
+    bool want = ni <= kCoopMaxInst && !(pc && std::string(pc) == "mg");
+    if (sizeof(Real) == 8 && std::getenv("APIC_SOLVER")) want = false;  // (asks for one of multigrid's two forms)
     for (const Inst& I : S->inst) want = want && !(I.flags & (APIC_NO_FIELD | APIC_BOLTZMANN));
     const char* dm = std::getenv("APIC_DIRECT");
     const std::string direct = dm ? dm : "auto";
-    // auto: the reduction where all its blocks (dense level 1) fit in L2
-    // (fewer, shorter phases), else nested dissection (its fronts stream
-    // about a tenth of the reduction's bytes from DRAM)
+    // auto: the reduction where every grid is small (its few phases are then
+    // shorter than the dissection's two sweeps over the tree) and all its
+    // blocks fit in L2, else the dissection (density, solve and fields, us:
+    // 64 x 32 61 and 91, 160 x 80 112 and 117, 192 x 96 138 and 124, 256 x 128
+    // 173 and 131, 96 x 200 188 and 122).  FP64 particles: the dissection (64 x
+    // 32 93 with multigrid's dense inverse and 66, 96 x 48 851 and 74)
     bool red_fits = false;
-    if (want && direct == "auto") {
+    if (want && direct == "auto" && sizeof(Real) == 4) {
       double b = 0.0;
       bool ok = true;
       for (int k = 0; k < ni && ok; ++k) {
         BcrInst B{};
-        ok = bcr_layout(S->inst[k], B, true);
+        ok = S->inst[k].nodes < 16384 && S->inst[k].N2 <= 97 && bcr_layout(S->inst[k], B, true);
         b += 4.0 * ((double)B.blocks * (double)B.blk + (double)B.tail_n * (double)B.tail_np);
       }
       red_fits = ok && b <= 112.0 * 1024 * 1024;
@@ -1010,16 +1018,101 @@ static int setup(apic_sim* S) {
         const char* e = std::getenv("APIC_ND_LEAF");
         leaf = e ? std::max(1, std::min(256, std::atoi(e))) : 16;
       }
-      if (!nd_build(I.n1 - 1, I.N2, nd_coef, &levels[k][0], leaf, T, false, nds[k], why) ||
+      if (!nd_build(I.n1 - 1, I.N2, nd_coef, &levels[k][0], leaf, T, sizeof(Real) == 8, nds[k], why) ||
           nds[k].depth > kNdMaxDepth)
         use_nd[k] = 0;  // the reduction (or multigrid) instead
     }
     long long off = 0;
+    // every instance by nested dissection: the dataflow solve (nd_solve.cu;
+    // APIC_ND_FLOW=0: one grid barrier per tree level instead, FP32 alone)
+    bool flow = want;
+    for (int k = 0; k < ni; ++k) flow = flow && use_nd[k];
+    if (const char* e = std::getenv("APIC_ND_FLOW")) flow = flow && std::atoi(e) != 0;
+    if (flow) {
+      int dev = 0, sms = 0;
+      cudaGetDevice(&dev);
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+      double nodes = 0.0;
+      for (int k = 0; k < ni; ++k) nodes += (double)S->inst[k].nodes;
+      bcr_in.assign(ni, BcrInst{});
+      std::vector<int64_t> words(ni + 1, 0);  // first word of each instance's records
+      for (int k = 0; k < ni && flow; ++k) {
+        const Inst& I = S->inst[k];
+        BcrInst& B = bcr_in[k];
+        NdLevels lvl;
+        const int f0 = (int)ndu.fronts.size();
+        nd_layout(nds[k], 0, nd_w, kNdWarpMaxS, kNdWarpMaxU, kNdWarpStage, kNdTaskFloats, kNdTaskRows, kNdTaskFronts,
+                  kNdUnitStage, 1, ndu, lvl);
+        const int nf = (int)ndu.fronts.size() - f0;
+        // the share of the CTAs by nodes (the sums do not depend on the tasks)
+        const int ctas = std::max(1, (int)std::lround(sms * (double)I.nodes / nodes));
+        const size_t t0 = nd_tasks.size();
+        for (int sw = 0; sw < 2 && flow; ++sw)
+          flow = nd_flow_tasks(ndu, f0, nf, nds[k].depth, k, sw == 0, kElem, nd_workers(kElem) * ctas, nd_vec_cap(kElem),
+                               kElem == 1 ? 4 * kNdUnits * ctas : 1 << 30, nd_tasks);
+        words[k + 1] = words[k];
+        for (size_t t = t0; t < nd_tasks.size(); ++t) {
+          nd_off.push_back(words[k + 1]);
+          words[k + 1] += nd_tasks[t].words;
+        }
+        flow = flow && words[k + 1] / 4 < (1ll << 31) && nd_w + nds[k].w_total < (1ll << 31);
+        nd_w += (nds[k].w_total + 63) & ~63ll;
+        B.nd = 1;
+        B.M = I.n1 - 1;
+        B.N = I.N2;
+        B.Np = (B.N + 3) & ~3;
+        B.nd_depth = nds[k].depth;
+        B.foff = bcr_rows;
+        bcr_rows += (long long)B.M * B.N;
+        B.node_off = I.node_off;
+        B.nodes = I.nodes;
+        B.st_off = I.lv[0].st;
+        nd_flow_places(ndu, f0, nf, (int64_t)B.M * B.N, nd_place, nd_perm);
+      }
+      flow = flow && bcr_rows + nd_w < (1ll << 31) && total_nodes < (1ll << 31);
+      if (flow) {
+        pl.bcr.nd_elem = kElem;
+        size_t fr = 0, tot = 0;
+        if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) fr = 0;
+        cudaGetLastError();
+        const double bytes = 4.0 * (double)words[ni];
+        pl.bcr.bytes = (int64_t)bytes;
+        flow = bytes <= kBcrMaxBytes && bytes <= 0.6 * (double)fr && (bcr_nb = nd_configure(pl, sms)) > 0;
+      }
+      if (flow) {
+        // forward from the deepest tree level, backward from the root: every
+        // record after those it reads from
+        std::vector<int> fe, be;
+        for (size_t t = 0; t < nd_tasks.size(); ++t) (nd_tasks[t].fwd ? fe : be).push_back((int)t);
+        auto key = [&](int t) {
+          const NdFlowTask& T = nd_tasks[t];
+          return std::make_pair(T.fwd ? nds[T.inst].depth - T.level : T.level, T.inst);
+        };
+        for (std::vector<int>* v : {&fe, &be}) {
+          std::stable_sort(v->begin(), v->end(), [&](int a, int b) { return key(a) < key(b); });
+          for (int t : *v)
+            nd_list.push_back(make_int4((int)(nd_off[t] / 4), 4 * nd_tasks[t].words, nd_tasks[t].inst, nd_tasks[t].kind));
+        }
+        pl.bcr.nd_nf = (int)fe.size();
+        pl.bcr.nd_nb = (int)be.size();
+        pl.bcr.nd_stream = 4.0 * (double)words[ni] > 96.0 * 1024 * 1024;  // (L2: 129 MB)
+      } else {  // a front beyond a record or a worker's vectors: level by level (FP32), multigrid (FP64)
+        pl.bcr.nd_elem = 0;
+        ndu = NdUpload();
+        nd_tasks.clear();
+        nd_off.clear();
+        nd_place.clear();
+        nd_perm.clear();
+        nd_w = 0;
+        bcr_rows = 0;
+      }
+    }
+    if (sizeof(Real) == 8) want = want && flow;
     // dense level-1 blocks when the whole reduction then still fits in L2
     // (fewer phases); else level 1 applies the stencil's couplings (fewer
     // bytes streamed from DRAM)
     const double l2_fit = 112.0 * 1024 * 1024;
-    for (int dense1 = 1; dense1 >= 0 && want; --dense1) {
+    for (int dense1 = 1; dense1 >= 0 && want && !flow; --dense1) {
       off = 0;
       bcr_rows = 0;
       bcr_in.assign(ni, BcrInst{});
@@ -1085,13 +1178,13 @@ static int setup(apic_sim* S) {
       if (4.0 * (double)off <= l2_fit) break;
     }
     const double bytes = 4.0 * (double)off;
-    if (want) {
+    if (want && !flow) {
       size_t fr = 0, tot = 0;
       if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) fr = 0;
       cudaGetLastError();
       want = bytes <= kBcrMaxBytes && bytes <= 0.6 * (double)fr;
     }
-    if (want) {
+    if (want && !flow) {
       int dev = 0, sms = 0;
       cudaGetDevice(&dev);
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1104,6 +1197,7 @@ static int setup(apic_sim* S) {
       std::vector<std::vector<std::pair<int, int>>> stages(ni);  // (kind << 8 | level, tasks)
       int phases = 0;
       for (int k = 0; k < ni; ++k) {
+        if (flow) continue;
         const BcrInst& B = bcr_in[k];
         auto& st = stages[k];
         const int M = B.M;
@@ -1137,59 +1231,16 @@ static int setup(apic_sim* S) {
           }
           bcr_pre[(size_t)p * (ni + 1) + k + 1] = bcr_pre[(size_t)p * (ni + 1) + k] + cnt;
         }
-      // node phases: partial sums over kBcrSub-node ranges of each instance
-      // (the same alone or in a batch), task_sub ranges per task, about two
-      // tasks per CTA or more
+      // node phases: partial sums over ranges of each instance's nodes (the same
+      // alone or in a batch)
       bcr_npre.assign(ni + 1, 0);
       for (int k = 0; k < ni; ++k)
-        bcr_npre[k + 1] = bcr_npre[k] + (int)((S->inst[k].nodes + kBcrSub - 1) / kBcrSub);
+        bcr_npre[k + 1] = bcr_npre[k] + (int)((S->inst[k].nodes + range_nodes(S->inst[k].nodes) - 1) / range_nodes(S->inst[k].nodes));
       pl.bcr.chunks = bcr_npre[ni];
       pl.bcr.rows = bcr_rows;
-      pl.bcr.task_sub = (int)std::max<long long>(1, std::min<long long>(kBcrMaxTaskSub, pl.bcr.chunks / (2ll * bcr_nb)));
-      bcr_tpre.assign(ni + 1, 0);
-      for (int k = 0; k < ni; ++k)
-        bcr_tpre[k + 1] = bcr_tpre[k] + (bcr_npre[k + 1] - bcr_npre[k] + pl.bcr.task_sub - 1) / pl.bcr.task_sub;
       pl.bcr.n_inst = ni;
       pl.bcr.phases = phases;
       pl.bcr.nd_wrows = nd_w;
-      // dataflow sweeps when every instance is solved by nested dissection
-      // (APIC_ND_FLOW=0: one grid barrier per tree level instead): a task
-      // waits only for the fronts it reads (forward: its fronts' children,
-      // backward: their parents), every front counting its finished tasks
-      bool all_nd = true;
-      for (int k = 0; k < ni; ++k) all_nd = all_nd && use_nd[k];
-      if (const char* e = std::getenv("APIC_ND_FLOW")) all_nd = all_nd && std::atoi(e) != 0;
-      pl.bcr.nd_flow = all_nd ? 1 : 0;
-      nd_flow.clear();
-      nd_need.clear();
-      if (all_nd) {
-        const int nf = (int)ndu.fronts.size();
-        nd_need.assign(2 * (size_t)nf, 0);
-        std::vector<std::pair<std::pair<int, int>, int2>> fe, be;  // ((key, instance), (task, instance))
-        for (int k = 0; k < ni; ++k) {
-          const BcrInst& B = bcr_in[k];
-          for (int l = 0; l <= B.nd_depth; ++l) {
-            for (int t = B.nd_ft[l]; t < B.nd_ft[l + 1]; ++t) fe.push_back({{B.nd_depth - l, k}, make_int2(t, k)});
-            for (int t = B.nd_bt[l]; t < B.nd_bt[l + 1]; ++t) be.push_back({{l, k}, make_int2(t, k)});
-          }
-        }
-        auto by_key = [](const std::pair<std::pair<int, int>, int2>& a, const std::pair<std::pair<int, int>, int2>& b) {
-          return a.first < b.first || (a.first == b.first && a.second.x < b.second.x);
-        };
-        std::stable_sort(fe.begin(), fe.end(), by_key);
-        std::stable_sort(be.begin(), be.end(), by_key);
-        for (int sw = 0; sw < 2; ++sw)
-          for (const auto& x : sw == 0 ? fe : be) {
-            nd_flow.push_back(x.second);
-            const NdTask& T = ndu.tasks[x.second.x];
-            if (T.warp == 0) nd_need[(size_t)sw * nf + T.front] += 1;
-            else
-              for (int q = 0; q < T.n; ++q) nd_need[(size_t)sw * nf + T.front + q] += 1;
-          }
-        pl.bcr.nd_nf = (int)fe.size();
-        pl.bcr.nd_nb = (int)be.size();
-        pl.bcr.nd_fronts = nf;
-      }
     } else {
       pl.bcr.n_inst = 0;
     }
@@ -1269,30 +1320,55 @@ static int setup(apic_sim* S) {
     // access-policy window covers them)
     d.bcr = (float*)A((size_t)pl.bcr.bytes);
     S->bcr_bytes = (size_t)pl.bcr.bytes;
-    d.bcr_f = (float*)A(sizeof(float) * kBcrMaxRhs * (size_t)bcr_rows);  // up to kBcrMaxRhs right-hand sides
-    d.bcr_e = (float*)A(sizeof(float) * kBcrMaxRhs * (size_t)bcr_rows);
+    const size_t E = pl.bcr.nd_elem == 2 ? sizeof(double) : sizeof(float);  // the corrections' type
+    d.bcr_f = (float*)A(E * kBcrMaxRhs * (size_t)bcr_rows);  // up to kBcrMaxRhs right-hand sides
+    d.bcr_e = (float*)A(E * kBcrMaxRhs * (size_t)bcr_rows);
     d.bcr_inst = (const BcrInst*)A(sizeof(BcrInst) * ni);
     d.bcr_kind = (const int32_t*)A(sizeof(int32_t) * bcr_kind.size());
     d.bcr_pre = (const int32_t*)A(sizeof(int32_t) * bcr_pre.size());
     d.bcr_npre = (const int32_t*)A(sizeof(int32_t) * bcr_npre.size());
-    d.bcr_tpre = (const int32_t*)A(sizeof(int32_t) * bcr_tpre.size());
-    d.bcr_part = (double*)A(sizeof(double) * (1 + kBcrMaxRhs) * (size_t)pl.bcr.chunks);
-    if (!ndu.fronts.empty()) {
+    d.bcr_part = (double*)A(sizeof(double) * ((1 + kBcrMaxRhs) * (size_t)pl.bcr.chunks +
+                                              2 * kBcrMaxRhs * (size_t)(pl.bcr.chunks + ni)));
+    if (pl.bcr.nd_elem > 0) {
+      d.nd_rec = (const unsigned char*)d.bcr;
+      d.nd_list = (const int4*)A(sizeof(int4) * nd_list.size());
+      d.nd_perm = (const int32_t*)A(sizeof(int32_t) * (size_t)bcr_rows);
+      d.nd_w = (float*)A(E * kBcrMaxRhs * (size_t)std::max<long long>(1, nd_w));
+      d.nd_e2 = A(E * kBcrMaxRhs * (size_t)bcr_rows);
+      if (S->status != APIC_OK) return S->status;
+      S->h2d((int4*)d.nd_list, nd_list.data(), nd_list.size());
+      S->h2d((int32_t*)d.nd_perm, nd_perm.data(), nd_perm.size());
+      // the records, instance by instance (the host copy of one at a time)
+      std::vector<int32_t> rec;
+      for (int k = 0, t0 = 0; k < ni; ++k) {
+        int t1 = t0;
+        while (t1 < (int)nd_tasks.size() && nd_tasks[t1].inst == k) ++t1;
+        const int64_t w0 = nd_off[t0], w1 = t1 < (int)nd_tasks.size() ? nd_off[t1] : pl.bcr.bytes / 4;
+        const NdFlowInst I{bcr_in[k].N, (int)bcr_in[k].foff, (int)bcr_in[k].node_off};
+        const NdFactor& F = nds[k];
+        rec.resize((size_t)(w1 - w0));
+        parallel_for(std::min(64, t1 - t0), [&](int q) {
+          for (int t = t0 + q; t < t1; t += std::min(64, t1 - t0)) {
+            int32_t* out = rec.data() + (nd_off[t] - w0);
+            if constexpr (sizeof(Real) == 8)
+              nd_flow_write<double>(ndu, nd_tasks[t], nd_place, nd_perm.data() + I.foff, I, F.fm64.data(), 0, F.nb64.data(), F.fm_total, out);
+            else
+              nd_flow_write<float>(ndu, nd_tasks[t], nd_place, nd_perm.data() + I.foff, I, F.fm.data(), 0,
+                                   F.nb.data(), F.fm_total, out);
+          }
+        });
+        S->h2d((int32_t*)d.bcr + w0, rec.data(), rec.size());
+        if (!S->sync()) return S->status;  // the host copies are reused or released below
+        nds[k] = NdFactor();
+        t0 = t1;
+      }
+    } else if (!ndu.fronts.empty()) {
       d.nd_front = (const NdFront*)A(sizeof(NdFront) * ndu.fronts.size());
       d.nd_idx = (const int32_t*)A(sizeof(int32_t) * ndu.idx.size());
       d.nd_gather = (const int32_t*)A(sizeof(int32_t) * ndu.gather.size());
       d.nd_task = (const int4*)A(sizeof(NdTask) * ndu.tasks.size());
       d.nd_w = (float*)A(sizeof(float) * kBcrMaxRhs * (size_t)std::max<long long>(1, nd_w));
-      if (pl.bcr.nd_flow) {
-        d.nd_flow = (const int2*)A(sizeof(int2) * nd_flow.size());
-        d.nd_need = (const int32_t*)A(sizeof(int32_t) * nd_need.size());
-        d.nd_done = (unsigned*)A(sizeof(unsigned) * 2 * kBcrMaxRhs * (size_t)pl.bcr.nd_fronts);
-      }
       if (S->status != APIC_OK) return S->status;
-      if (pl.bcr.nd_flow) {
-        S->h2d((int2*)d.nd_flow, nd_flow.data(), nd_flow.size());
-        S->h2d((int32_t*)d.nd_need, nd_need.data(), nd_need.size());
-      }
       S->h2d((NdFront*)d.nd_front, ndu.fronts.data(), ndu.fronts.size());
       S->h2d((int32_t*)d.nd_idx, ndu.idx.data(), ndu.idx.size());
       S->h2d((int32_t*)d.nd_gather, ndu.gather.data(), ndu.gather.size());
@@ -1340,13 +1416,12 @@ static int setup(apic_sim* S) {
     S->h2d((int32_t*)d.bcr_kind, bcr_kind.data(), bcr_kind.size());
     S->h2d((int32_t*)d.bcr_pre, bcr_pre.data(), bcr_pre.size());
     S->h2d((int32_t*)d.bcr_npre, bcr_npre.data(), bcr_npre.size());
-    S->h2d((int32_t*)d.bcr_tpre, bcr_tpre.data(), bcr_tpre.size());
     if (!S->sync()) return S->status;
     std::vector<float> blocks;
     std::vector<double> T, aug;
     for (int k = 0; k < ni; ++k) {
       const BcrInst& B = bcr_in[k];
-      if (B.nd) continue;
+      if (B.nd || pl.bcr.nd_elem > 0) continue;
       if (!bcr_factor(levels[k][0], B, blocks, T))
         return S->fail(APIC_ERR_INVALID_ARG, "block cyclic reduction: singular diagonal block");
       if (B.blocks > 0) S->h2d(d.bcr + B.base, blocks.data(), (size_t)(B.blocks * B.blk));
@@ -1894,7 +1969,8 @@ extern "C" int apic_stats(apic_sim* S, apic_stats_t* out) {
                                                                : push_window_rows<float>(S->max_n2));
   out->chunk_group = S->chunk_group > 0 ? S->chunk_group : 4;
   out->chunk_items = S->precision == APIC_FP64 ? 0 : (S->chunk_items > 0 ? S->chunk_items : push4_default_items(S));
-  out->solver = S->plan.bcr.n_inst > 0 ? (S->d.nd_front ? APIC_SOLVER_ND : APIC_SOLVER_BCR)
+  out->solver = S->plan.bcr.nd_elem == 2 ? APIC_SOLVER_ND64
+                : S->plan.bcr.n_inst > 0 ? (S->plan.bcr.nd_elem > 0 || S->d.nd_front ? APIC_SOLVER_ND : APIC_SOLVER_BCR)
                                        : (S->coop > 0 ? APIC_SOLVER_MG_COOP : APIC_SOLVER_MG_KERNELS);
   out->sorts = S->sorts;
   out->kernels_per_sort = 6;

@@ -183,9 +183,9 @@ struct DevPtrs {
   const BcrInst* bcr_inst;        // [n_inst]
   const int32_t* bcr_kind;        // [phases][n_inst]: kind << 8 | level of instance k's tasks in a phase (0: none)
   const int32_t* bcr_pre;         // [phases][n_inst + 1]: prefix sums of the instances' task counts
-  const int32_t* bcr_npre;        // [n_inst + 1]: prefix sums of the instances' partial-sum ranges (kBcrSub nodes)
-  const int32_t* bcr_tpre;        // [n_inst + 1]: prefix sums of the instances' node tasks
-  double* bcr_part;               // [1 + kBcrMaxRhs][chunks]: |b|^2, then |r|^2 per right-hand side, of each range
+  const int32_t* bcr_npre;        // [n_inst + 1]: prefix sums of the instances' partial-sum ranges (range_nodes)
+  double* bcr_part;               // [1 + kBcrMaxRhs][chunks]: |b|^2, then |r|^2 per right-hand side, of each range,
+                                  // then two areas of their segments' sums [kBcrMaxRhs * (chunks + n_inst)]
   // nested dissection (instances with BcrInst::nd): fronts of every such
   // instance (offsets global: idx, gather, matrices in bcr, update vectors
   // per right-hand side in nd_w), their index and gather tables, the tasks
@@ -196,13 +196,15 @@ struct DevPtrs {
   const int4* nd_task;
   const longlong2* nd_trange;  // per task: its matrix floats [x, y) in bcr (one contiguous range)
   float* nd_w;
-  // dataflow sweeps (BcrPlan::nd_flow): the forward then the backward task
-  // order (task, instance; every task after the tasks it depends on), the
-  // tasks each front takes per sweep [2][fronts] and the done counters
-  // [2][kBcrMaxRhs][fronts]
-  const int2* nd_flow;
-  const int32_t* nd_need;
-  unsigned* nd_done;
+  // dataflow sweeps (BcrPlan::nd_elem > 0; bcr_f, bcr_e and nd_w then hold the
+  // sweeps' type): the task records (nd_records.h), the forward then the
+  // backward list of them (offset in 16-byte units, bytes, instance, kind;
+  // every record after those it reads from), and the backward sweep's result,
+  // [kBcrMaxRhs][rows]
+  const unsigned char* nd_rec;
+  const int32_t* nd_perm;        // [rows]: place of an instance's unknown in bcr_f and bcr_e (front by front)
+  const int4* nd_list;
+  void* nd_e2;
 };
 
 #ifdef __CUDACC__
@@ -362,8 +364,9 @@ constexpr int kBcrMaxNWide = 544;   // the wide one (17 outputs per lane): grids
 constexpr int kBcrTailMax = 2048;
 constexpr double kBcrMaxBytes = 24.0 * 1024 * 1024 * 1024;  // FP32 blocks of a whole batch held on the device
 constexpr int kBcrUpdRows = 4;       // level-1 kept rows per update task
-constexpr int kBcrSub = 256;         // nodes per partial sum of the node phases (density, residual)
-constexpr int kBcrMaxTaskSub = 8;    // partial-sum ranges per node task at most
+// Nodes per partial sum of the node phases (density, residual), one warp's
+// task: a node per lane on small grids, two on others.
+__host__ __device__ constexpr int range_nodes(long long nodes) { return nodes <= 8192 ? 32 : 64; }
 // task kinds of a phase of one instance
 constexpr int kBcrFwd1 = 1;   // y_k = B_k^-1 f_k, level-1 eliminated rows
 constexpr int kBcrUpd1 = 2;   // f_i -= A_i y_{i-1} + C_i y_{i+1}, level-1 kept rows
@@ -433,16 +436,14 @@ struct BcrPlan {
   int wide;                 // solve kernel: 0 narrow reduction, 1 wide reduction (some block larger than
                             // kBcrMaxN, or reduction and nested dissection), 2 nested dissection alone
   int64_t bytes;            // device bytes of all blocks and tail inverses
-  int64_t chunks;           // partial-sum ranges of all instances (kBcrSub nodes each)
+  int64_t chunks;           // partial-sum ranges of all instances (range_nodes)
   int64_t rows;             // floats of one right-hand side's rows in bcr_f / bcr_e (all instances)
-  int task_sub;             // partial-sum ranges per node task (1..kBcrMaxTaskSub)
-  int pad2;
   int64_t nd_wrows;         // floats of one right-hand side's update vectors in nd_w (all instances)
   int nd_floats;            // shared-memory floats a large nested-dissection front needs (0: none)
-  int nd_flow;              // 1: every instance by nested dissection, each sweep one dataflow phase
-  int nd_nf, nd_nb;         // entries of the forward and backward task orders
-  int nd_fronts;            // fronts of all instances
-  int pad3;
+  int nd_elem;              // > 0: every instance by nested dissection, each sweep one dataflow phase (nd_solve.cu),
+                            // in FP32 (1) or FP64 (2: words per matrix element)
+  int nd_nf, nd_nb;         // entries of the forward and backward record lists
+  int nd_stream;            // 1: the records exceed L2 by far (copied with an evict-first hint)
 };
 
 // Poisson (poisson.cu): host-side launch plan of the multigrid levels.
@@ -505,6 +506,14 @@ cudaError_t launch_solve_bcr_rhs(const DevPtrs& d, const SolvePlan& plan, int bl
 // and tail chunk, and the kernel's shared memory (plan.bcr.smem, plan.bcr.dyn).
 int bcr_configure(SolvePlan& plan, BcrInst* inst, int n_inst, int sms);
 const void* bcr_kernel(const SolvePlan& plan);  // the solve kernel (to find its graph node)
+// The dataflow solve (nd_solve.cu): its kernel, the CTAs of a launch (0: not
+// co-residable; sets plan.bcr.dyn) and the longest vector of a front it takes
+const void* nd_kernel(const SolvePlan& plan);
+int nd_configure(SolvePlan& plan, int sms);
+int nd_vec_cap(int elem);
+// Workers of 128 threads per CTA of the dataflow solve.
+constexpr int nd_workers(int elem) { return elem == 2 ? 4 : 6; }
+constexpr int nd_threads(int elem) { return 128 * nd_workers(elem); }
 // blocks CTAs (all resident) wait at a barrier that never completes, each
 // for d.wait_ns; d.bar must point at a zeroed counter of its own.
 void launch_wait_check(const DevPtrs& d, int blocks, cudaStream_t s);

@@ -29,12 +29,12 @@ namespace {
 #include "solver_common.cuh"
 #include "fields_common.cuh"
 #include "bulk_copy.cuh"
+#include "solve_nodes.cuh"
 
 constexpr int kBcrThreads = 512;
 constexpr int kBcrWarps = kBcrThreads / 32;
 constexpr int kTailChunk = 16;      // tail rows per task at most (one per warp)
 constexpr int kUpdRows = kBcrUpdRows;
-constexpr int kRangesPerPass = kBcrThreads / kBcrSub;  // partial-sum ranges a CTA covers at once
 // shared memory of the nested-dissection tasks (the wide kernel's reduction
 // buffer, kBcrWarps x kBcrMaxNWide floats): a large front's vector
 // (kNdVecCap floats) and its task's rows after it; a small front's v_S, z_S
@@ -48,7 +48,6 @@ constexpr int kNdWarpArea = 8 * kNdWarpMaxS;   // 512 floats
 constexpr int kNdTinyArea = 8 * kNdTinyS;      // 128 floats, four groups per warp
 static_assert(kNdWarpMaxU == 3 * kNdWarpMaxS && kNdTinyU == 3 * kNdTinyS, "area layout");
 static_assert(kNdWarpArea <= kBcrMaxNWide && 4 * kNdTinyArea <= kNdWarpArea && kNdTinyArea % 4 == 0, "areas");
-static_assert(kRangesPerPass * kBcrSub == kBcrThreads, "whole ranges per pass");
 
 // res = sum_t M_t v_t for NT column-major blocks (column stride Np) and
 // vectors v_t in shared memory, by the whole CTA: warp w takes the columns
@@ -138,17 +137,6 @@ __device__ bool run_task(Ctx& c, const BcrInst& B, const float* const* src, cons
     task_mv<NT, false, kMC>(src, vt, B.N, B.Np, c.red, c.sres);
   }
   return true;
-}
-
-// Instance of task t of a phase: pre[k] <= t < pre[k + 1] (prefix in shared memory).
-__device__ __forceinline__ int task_inst_s(const int* pre, int ni, int t) {
-  int lo = 0, hi = ni - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (pre[mid] <= t) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
 }
 
 // Blocks (or tail rows) read by task q of kind `kind` at level l of instance
@@ -543,54 +531,15 @@ __device__ __forceinline__ void nd_back_store(const DevPtrs& d, const NdFront& F
 // by one bulk copy issued before the vectors are gathered; the vectors live in the wide kernel's
 // reduction buffer (a large front's at [0, kNdVecCap) and its task rows'
 // values after it; kNdWarpArea floats per warp, kNdTinyArea per 8-lane group).
-// A nested-dissection worker: the whole CTA (barrier 0), or one half of it
-// (named barriers 1 and 2, 256 threads each) in the dataflow sweeps, so that
-// an SM has two tasks in flight.  Its vectors, stage and copy barrier are its
-// own.
+// A nested-dissection worker: the whole CTA.
 struct NdUnit {
   int t, n, nw;   // thread within the unit, threads, warps
-  int id;         // named barrier (0: __syncthreads)
   float* red;     // the unit's vector areas
   float* sbuf;    // the unit's matrix stage
   uint64_t* bar;  // the unit's copy barrier
   int vcap;       // floats of a large front's vector; its task rows' values follow
-  __device__ __forceinline__ void sync() const {
-    if (id == 0) __syncthreads();
-    else asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
-  }
-  __device__ __forceinline__ bool sync_and(bool p) const {
-    if (id == 0) return __syncthreads_and(p) != 0;
-    unsigned r;
-    asm volatile(
-        "{\n .reg .pred pi, po;\n setp.ne.u32 pi, %1, 0;\n bar.red.and.pred po, %2, %3, pi;\n"
-        " selp.u32 %0, 1, 0, po;\n}\n"
-        : "=r"(r)
-        : "r"((unsigned)p), "r"(id), "r"(n)
-        : "memory");
-    return r != 0;
-  }
+  __device__ __forceinline__ void sync() const { __syncthreads(); }
 };
-
-// mbar_wait for a unit's copies (every thread of the unit).
-__device__ bool nd_mbar_wait(const NdUnit& U, uint64_t* bar, unsigned parity, int32_t* err) {
-  bool ok = false;
-  for (long long k = 0; k < (1ll << 22); ++k) {
-    if (mbar_try_wait(bar, parity)) {
-      ok = true;
-      break;
-    }
-    if ((k & 1023) == 1023 && ((*(volatile int32_t*)err) & kErrTimeout)) break;
-    __nanosleep(32);
-  }
-  if (!ok) {
-    atomicOr(err, kErrTimeout);
-    for (long long k = 0; k < (1ll << 22); ++k) {
-      if (mbar_try_wait(bar, parity)) break;
-      __nanosleep(64);
-    }
-  }
-  return U.sync_and(ok);
-}
 
 // Issue the bulk copy of task `tr`'s matrix rows into the unit's stage (its
 // thread 0; after the unit's earlier reads of the stage).
@@ -602,10 +551,8 @@ __device__ __forceinline__ void nd_issue(const DevPtrs& d, const NdUnit& U, cons
   }
 }
 
-// issued: the task's copy was issued before (nd_issue), e.g. while its
-// dependencies were awaited.
 __device__ bool run_nd_task(const DevPtrs& d, Ctx& c, const NdUnit& U, const BcrInst& B, int kind, const int4 T,
-                            const longlong2 tr, bool issued, float* fb, float* eb, double* xb, float* wb) {
+                            const longlong2 tr, float* fb, float* eb, double* xb, float* wb) {
   const float* f = fb + B.foff;
   float* e = eb + B.foff;
   double* x = xb + B.node_off;
@@ -621,12 +568,12 @@ __device__ bool run_nd_task(const DevPtrs& d, Ctx& c, const NdUnit& U, const Bcr
     return true;
   }
   const bool staged = m1 > m0;
-  if (!issued) nd_issue(d, U, tr);
+  nd_issue(d, U, tr);
   // matrix float o of the buffer in the stage
   auto at = [&](long long o) { return U.sbuf + (o - m0); };
   auto wait = [&]() {
     if (!staged) return true;
-    if (!nd_mbar_wait(U, U.bar, c.parity, c.err)) return false;
+    if (!mbar_wait(U.bar, c.parity, c.err)) return false;
     c.parity ^= 1u;
     return true;
   };
@@ -787,145 +734,8 @@ __device__ bool run_nd_task(const DevPtrs& d, Ctx& c, const NdUnit& U, const Bcr
 __device__ __forceinline__ bool run_nd(const DevPtrs& d, Ctx& c, const BcrInst& B, int kind, int l, int q, float* fb,
                                        float* eb, double* xb, float* wb) {
   const int t = (kind == kNdFwd ? B.nd_ft[l] : B.nd_bt[l]) + q;
-  const NdUnit U{(int)threadIdx.x, (int)blockDim.x, kBcrWarps, 0, c.red, c.sbuf, c.bar, kNdVecCap};
-  return run_nd_task(d, c, U, B, kind, d.nd_task[t], d.nd_trange[t], false, fb, eb, xb, wb);
-}
-
-// ---- dataflow sweeps (BcrPlan::nd_flow) ----
-// CTA b takes the sweep's tasks b, b + nb, ... of the task order (right-hand
-// side by right-hand side).  Before a task runs, thread f of the CTA
-// waits until front f of the task has what it reads: forward, both children
-// have finished all their tasks; backward, the parent has.  After the task,
-// each of its fronts counts one finished task (release; the waits acquire).
-// The order puts every task after those it waits for, every CTA runs its
-// tasks in order and every CTA is resident (cooperative launch), so the
-// earliest unfinished task always runs.  A wait gives up after d.wait_ns (kErrTimeout): false.
-__device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-
-__device__ bool nd_wait_deps(const DevPtrs& d, const BcrPlan& pl, const NdUnit& U, int kind, int rh, const int4 T) {
-  const int nfr = T.w == 0 ? 1 : T.z;
-  const int sw = kind == kNdFwd ? 0 : 1;
-  const unsigned* done = d.nd_done + ((long long)sw * kBcrMaxRhs + rh) * pl.nd_fronts;
-  const int32_t* need = d.nd_need + (long long)sw * pl.nd_fronts;
-  bool ok = true;
-  if (U.t < nfr) {
-    const NdFront& F = d.nd_front[T.x + U.t];
-    int dep[2] = {-1, -1};
-    if (kind == kNdFwd) {
-      dep[0] = F.child[0];
-      dep[1] = F.child[1];
-    } else {
-      dep[0] = F.parent;
-    }
-    unsigned long long t0 = 0;
-    for (int q = 0; q < 2 && ok; ++q) {
-      if (dep[q] < 0) continue;
-      const unsigned want = (unsigned)need[dep[q]];
-      for (long long spins = 0; ld_acquire_u32(done + dep[q]) < want; ++spins) {
-        if ((spins & 63) == 63) {
-          if ((*(volatile int*)d.err) & kErrTimeout) {
-            ok = false;
-            break;
-          }
-          const unsigned long long now = global_ns();
-          if (t0 == 0) t0 = now;
-          else if (now - t0 > d.wait_ns) {
-            atomicOr(d.err, kErrTimeout);
-            ok = false;
-            break;
-          }
-        }
-        __nanosleep(64);
-      }
-    }
-  }
-  return U.sync_and(ok);
-}
-
-// After a task (its last unit barrier behind it): each front counts one.
-__device__ __forceinline__ void nd_signal(const DevPtrs& d, const BcrPlan& pl, const NdUnit& U, int kind, int rh,
-                                          const int4 T) {
-  const int nfr = T.w == 0 ? 1 : T.z;
-  const int sw = kind == kNdFwd ? 0 : 1;
-  if (U.t < nfr) {
-    unsigned* p = d.nd_done + ((long long)sw * kBcrMaxRhs + rh) * pl.nd_fronts + T.x + U.t;
-    __threadfence();
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p) : "memory");
-  }
-}
-
-// Fixed-order sum of part[r chunks + npre[k] .. r chunks + npre[k+1]) for
-// every system v = r ni + k (right-hand side r < nrhs, instance k) with
-// sel[v] (all when sel is null), one warp per system; out[v] in shared
-// memory, the same in every CTA.
-__device__ void inst_sums(const double* part, const int* npre, int ni, int nrhs, long long chunks, const int* sel,
-                          double* out) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int v = warp; v < nrhs * ni; v += kBcrWarps) {
-    if (sel && !sel[v]) continue;
-    const int r = v / ni, k = v - r * ni;
-    const double* pr = part + (long long)r * chunks;
-    double x = 0.0;
-    for (int c = npre[k] + lane; c < npre[k + 1]; c += 32) x += pr[c];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(kFull, x, o);
-    if (lane == 0) out[v] = x;
-  }
-  __syncthreads();
-}
-
-// Node tasks over the ranges of kBcrSub nodes of every instance (range c of
-// instance k: nodes c kBcrSub .. (c + 1) kBcrSub - 1).  A task covers tsub
-// consecutive ranges of one instance, kRangesPerPass per pass of the CTA; the tasks of
-// all instances (and right-hand sides r < nrhs) are spread over the CTAs.
-// body(r, k, I, nd) returns the node's contribution to its range's sum,
-// which goes to part[r chunks + npre[k] + c] (when part
-// is not null) as a warp-shuffle tree per warp and the range's warps in order: the
-// sums do not depend on the task size, the CTA or the other instances of a
-// batch.  ws: kBcrMaxTaskSub / kRangesPerPass * kBcrWarps doubles of shared memory.
-template <class F>
-__device__ void node_tasks(const DevPtrs& d, const int* npre, const int* tpre, int tsub, int nrhs, long long chunks,
-                           const int* sel, double* part, double* ws, F body) {
-  constexpr int kPasses = kBcrMaxTaskSub / kRangesPerPass;
-  const int ni = d.n_inst, nb = gridDim.x;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int half = threadIdx.x / kBcrSub, r = threadIdx.x % kBcrSub;  // range within the pass, node within it
-  const int per_rhs = tpre[ni], total = nrhs * per_rhs;
-  for (int t = blockIdx.x; t < total; t += nb) {
-    const int rh = t / per_rhs, tt = t - rh * per_rhs;
-    const int k = task_inst_s(tpre, ni, tt);
-    if (sel && !sel[rh * ni + k]) continue;
-    const Inst& I = d.inst[k];
-    const int s0 = (tt - tpre[k]) * tsub, s1 = min(npre[k + 1] - npre[k], s0 + tsub);
-    double v[kPasses];
-#pragma unroll
-    for (int u = 0; u < kPasses; ++u) {
-      const int sc = s0 + kRangesPerPass * u + half;
-      const long long nd = (long long)sc * kBcrSub + r;
-      v[u] = sc < s1 && nd < I.nodes ? body(rh, k, I, nd) : 0.0;
-    }
-    if (!part) continue;
-#pragma unroll
-    for (int u = 0; u < kPasses; ++u) {
-      if (s0 + kRangesPerPass * u >= s1) break;
-      double x = v[u];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(kFull, x, o);
-      if (lane == 0) ws[u * kBcrWarps + warp] = x;
-    }
-    __syncthreads();
-    if (threadIdx.x < s1 - s0) {
-      const int i = threadIdx.x, u = i / kRangesPerPass, w0 = (i % kRangesPerPass) * (kBcrSub / 32);
-      double sum = 0.0;
-      for (int w = w0; w < w0 + kBcrSub / 32; ++w) sum += ws[u * kBcrWarps + w];
-      part[(long long)rh * chunks + npre[k] + s0 + i] = sum;
-    }
-    __syncthreads();
-  }
+  const NdUnit U{(int)threadIdx.x, (int)blockDim.x, kBcrWarps, c.red, c.sbuf, c.bar, kNdVecCap};
+  return run_nd_task(d, c, U, B, kind, d.nd_task[t], d.nd_trange[t], fb, eb, xb, wb);
 }
 
 // mode: kBcrRho = the step's density, initial guess and right-hand side are
@@ -950,12 +760,11 @@ __global__ void __launch_bounds__(kBcrThreads, 1) k_solve_bcr(DevPtrs d, BcrPlan
   __shared__ double s_rn[kCoopMaxInst];
   __shared__ int s_act[kCoopMaxInst];
   __shared__ int s_npre[kCoopMaxInst + 1];
-  __shared__ int s_tpre[kCoopMaxInst + 1];
-  __shared__ double s_ws[kBcrMaxTaskSub / kRangesPerPass * kBcrWarps];
+  __shared__ double s_seg[kSumSlots];
+  __shared__ int s_sp[kCoopMaxInst + 1];
   __shared__ int s_pre[kCoopMaxInst + 1];
   __shared__ int s_kind[kCoopMaxInst];
   __shared__ __align__(8) uint64_t s_bar;
-  __shared__ __align__(8) uint64_t s_ubar[kNdUnits];  // the workers' copy barriers (dataflow sweeps)
   __shared__ __align__(16) BcrInst s_b0;  // instance 0's table (one load per kernel instead of one per task)
   const int nb = gridDim.x, ni = d.n_inst, R = rhs.n, nv = R * ni;
   static_assert(kBcrMaxRhs == 3, "selections below");
@@ -966,14 +775,12 @@ __global__ void __launch_bounds__(kBcrThreads, 1) k_solve_bcr(DevPtrs d, BcrPlan
   Ctx c{s_dyn, &s_bar, 0u, red, sres, d.err};
   double* part_b = d.bcr_part;                           // |b|^2 per range
   double* part_r = d.bcr_part + pl.chunks;  // |r|^2 per range and right-hand side ([kBcrMaxRhs][chunks])
+  double* seg_sums = d.bcr_part + (1 + kBcrMaxRhs) * pl.chunks;
   for (int k = threadIdx.x; k <= ni; k += blockDim.x) {
     s_npre[k] = d.bcr_npre[k];
-    s_tpre[k] = d.bcr_tpre[k];
   }
-  const int tsub = pl.task_sub;
   for (int v = threadIdx.x; v < nv; v += blockDim.x) s_act[v] = only < 0 || v % ni == only;
   if (threadIdx.x == 0) mbar_init(&s_bar, 1);
-  if (threadIdx.x < kNdUnits) mbar_init(&s_ubar[threadIdx.x], 1);
   for (int w = threadIdx.x; w < (int)(sizeof(BcrInst) / 4); w += blockDim.x)
     ((int*)&s_b0)[w] = ((const int*)d.bcr_inst)[w];
   // this thread's entries of the next phase's task tables, loaded before a
@@ -992,15 +799,16 @@ __global__ void __launch_bounds__(kBcrThreads, 1) k_solve_bcr(DevPtrs d, BcrPlan
     }
   };
   __syncthreads();
+  sum_prefix(s_npre, ni, s_sp);
+  __syncthreads();
   if (mode & kBcrRho) {
     // rho, the initial guess and b at every node; |b|^2 per instance
-    node_tasks(d, s_npre, s_tpre, tsub, 1, pl.chunks, nullptr, part_b, s_ws,
-               [&](int, int k, const Inst& I, long long nd) {
-                 const double bv = rho_node(d, I, k, nd);
-                 return bv * bv;
-               });
+    node_tasks(d, s_npre, 1, pl.chunks, nullptr, part_b, nullptr, [&](int, int k, const Inst& I, int nd) {
+      const double bv = rho_node(d, I, k, nd);
+      return make_double2(bv * bv, 0.0);
+    });
     if (!grid_sync(d, nb)) return;
-    inst_sums(part_b, s_npre, ni, 1, pl.chunks, nullptr, s_bn);
+    if (!inst_sums(d, part_b, seg_sums, s_npre, s_sp, 1, pl.chunks, nullptr, s_bn, s_seg)) return;
   } else {
     // |b|^2 from the right-hand-side kernels' partials (fixed order)
     for (int v = threadIdx.x; v < nv; v += blockDim.x) {
@@ -1016,10 +824,10 @@ __global__ void __launch_bounds__(kBcrThreads, 1) k_solve_bcr(DevPtrs d, BcrPlan
   for (int it = 0;; ++it) {
     // FP64 residual of every instance still iterating, stored as the FP32
     // right-hand side of its reduction
-    node_tasks(d, s_npre, s_tpre, tsub, R, pl.chunks, s_act, part_r, s_ws,
-               [&](int rh, int k, const Inst& I, long long nd) {
+    node_tasks(d, s_npre, R, pl.chunks, s_act, part_r, nullptr,
+               [&](int rh, int k, const Inst& I, int nd) {
                  const int N = I.N2;
-                 const int i = (int)(nd / N), j = (int)(nd % N);
+                 const int i = nd / N, j = nd - i * N;
                  double rr = 0.0;
                  if (i > 0 && i < I.n1) {
                    const double r = b_of(rh)[I.node_off + nd] -
@@ -1028,19 +836,12 @@ __global__ void __launch_bounds__(kBcrThreads, 1) k_solve_bcr(DevPtrs d, BcrPlan
                    d.bcr_f[rh * pl.rows + d.bcr_inst[k].foff + (long long)(i - 1) * N + j] = (float)r;
                    rr = r * r;
                  }
-                 return rr;
+                 return make_double2(rr, 0.0);
                });
-    if constexpr ((kParts & 2) != 0) {
-      if (pl.nd_flow) {  // the dataflow sweeps' counters, for this pass
-        const long long nz = 2ll * kBcrMaxRhs * pl.nd_fronts;
-        for (long long z = (long long)blockIdx.x * blockDim.x + threadIdx.x; z < nz; z += (long long)nb * blockDim.x)
-          d.nd_done[z] = 0u;
-      }
-    }
     load_tab(0);
     if (!grid_sync(d, nb)) return;
     store_tab();  // read after the synchronisation that ends inst_sums
-    inst_sums(part_r, s_npre, ni, R, pl.chunks, s_act, s_rn);
+    if (!inst_sums(d, part_r, seg_sums, s_npre, s_sp, R, pl.chunks, s_act, s_rn, s_seg)) return;
     int more = 0;
     for (int v = threadIdx.x; v < nv; v += blockDim.x) {
       if (!s_act[v]) continue;
@@ -1064,52 +865,6 @@ __global__ void __launch_bounds__(kBcrThreads, 1) k_solve_bcr(DevPtrs d, BcrPlan
       }
     }
     if (!__syncthreads_or(more)) break;
-    if constexpr (kParts == 2) {
-      if (pl.nd_flow) {  // nested dissection of every instance: one dataflow phase per sweep
-        for (int sw = 0; sw < 2; ++sw) {
-          const int kind = sw == 0 ? kNdFwd : kNdBack;
-          const int n = sw == 0 ? pl.nd_nf : pl.nd_nb;
-          const int2* list = d.nd_flow + (sw == 0 ? 0 : pl.nd_nf);
-          const long long total = (long long)R * n;
-          // unit u (two per CTA) takes tasks u, u + 2 nb, ... (each after
-          // the tasks it waits for); the next task's entry is loaded while
-          // this one runs
-          constexpr int UT = kBcrThreads / kNdUnits, UW = kBcrWarps / kNdUnits;
-          const int h = (int)threadIdx.x / UT;
-          const NdUnit U{(int)threadIdx.x - h * UT, UT, UW, kNdUnits == 1 ? 0 : 1 + h, red + h * UW * MAXN,
-                         s_dyn + h * kNdUnitStage, s_ubar + h, UW * MAXN - kNdTaskRows};
-          const long long u0 = (long long)kNdUnits * blockIdx.x + h, nu = (long long)kNdUnits * nb;
-          auto entry = [&](long long t) { return list[t - (t / n) * n]; };
-          int2 en = u0 < total ? entry(u0) : make_int2(0, 0);
-          int4 T = u0 < total ? d.nd_task[en.x] : make_int4(0, 0, 0, 0);
-          bool good = true;
-          for (long long t = u0; t < total && good; t += nu) {
-            const int rh = (int)(t / n);
-            const long long tn = t + nu;
-            const int2 en_n = tn < total ? entry(tn) : en;
-            if (s_act[rh * ni + en.y]) {
-              // the matrix rows are static: their copy runs while the
-              // dependencies are awaited
-              const longlong2 tr = d.nd_trange[en.x];
-              nd_issue(d, U, tr);
-              good = nd_wait_deps(d, pl, U, kind, rh, T);
-              const BcrInst& B = en.y == 0 ? s_b0 : d.bcr_inst[en.y];
-              if (good)
-                good = run_nd_task(d, c, U, B, kind, T, tr, true, d.bcr_f + rh * pl.rows, d.bcr_e + rh * pl.rows,
-                                   x_of(rh), d.nd_w + rh * pl.nd_wrows);
-              if (good) nd_signal(d, pl, U, kind, rh, T);
-            }
-            en = en_n;
-            if (tn < total) T = d.nd_task[en.x];
-          }
-          // (a unit that gave up goes on to the grid barrier, which sees the
-          // time-out bit and ends the kernel)
-          if (!grid_sync(d, nb)) return;
-        }
-        if (blockIdx.x == 0 && threadIdx.x == 0) d.cnt[0] += 1;
-        continue;
-      }
-    }
     // the reduction passes: phase p runs the p-th stage of every instance
     for (int p = 0; p < pl.phases; ++p) {
       if (p > 0) {  // the phase's task tables (loaded before the last barrier)
@@ -1142,10 +897,10 @@ __global__ void __launch_bounds__(kBcrThreads, 1) k_solve_bcr(DevPtrs d, BcrPlan
   }
   if (mode & kBcrFields) {
     // phi is final everywhere (the last pass ended at a grid barrier)
-    node_tasks(d, s_npre, s_tpre, tsub, 1, pl.chunks, nullptr, nullptr, s_ws,
-               [&](int, int, const Inst& I, long long nd) {
+    node_tasks(d, s_npre, 1, pl.chunks, nullptr, nullptr, nullptr,
+               [&](int, int, const Inst& I, int nd) {
                  grad_node<float, float2>(d, I, nd);
-                 return 0.0;
+                 return make_double2(0.0, 0.0);
                });
     for (int k = nb - 1 - (int)blockIdx.x; k < ni; k += nb) surface_block(d, k, sh);
   }
@@ -1153,7 +908,7 @@ __global__ void __launch_bounds__(kBcrThreads, 1) k_solve_bcr(DevPtrs d, BcrPlan
 
 constexpr int static_smem(int maxn) {
   return 40 * 8 + 3 * maxn * 4 + maxn * 4 + kBcrWarps * maxn * 4 + kCoopMaxInst * 36 + 12 +
-         kBcrMaxTaskSub / kRangesPerPass * kBcrWarps * 8 + (int)sizeof(BcrInst) + 16 + 64;
+         kSumSlots * 8 + (kCoopMaxInst + 1) * 4 + (int)sizeof(BcrInst) + 16 + 64;
 }
 
 const void* kernel_for(const BcrPlan& b) {
@@ -1171,7 +926,7 @@ __global__ void k_wait_check(DevPtrs d) { grid_sync(d, gridDim.x + 1u); }
 
 }  // namespace
 
-const void* bcr_kernel(const SolvePlan& pl) { return kernel_for(pl.bcr); }
+const void* bcr_kernel(const SolvePlan& pl) { return pl.bcr.nd_elem > 0 ? nd_kernel(pl) : kernel_for(pl.bcr); }
 
 void launch_wait_check(const DevPtrs& d, int blocks, cudaStream_t s) { k_wait_check<<<blocks, 32, 0, s>>>(d); }
 
@@ -1245,7 +1000,8 @@ static cudaError_t launch_bcr(const DevPtrs& d, const SolvePlan& pl, int blocks,
   BcrRhs rr = rhs;
   int mm = mode, oo = only;
   void* args[] = {&dd, &pp, &mm, &oo, &rr};
-  return cudaLaunchCooperativeKernel(kernel_for(pl.bcr), dim3(blocks), dim3(kBcrThreads), args,
+  return cudaLaunchCooperativeKernel(bcr_kernel(pl), dim3(blocks),
+                                     dim3(pl.bcr.nd_elem > 0 ? nd_threads(pl.bcr.nd_elem) : kBcrThreads), args,
                                      (size_t)pl.bcr.dyn, s);
 }
 

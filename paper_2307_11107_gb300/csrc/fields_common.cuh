@@ -16,7 +16,7 @@
 __device__ __forceinline__ double rho_node(const DevPtrs& d, const Inst& I, int inst, long long nd) {
   const long long g = I.node_off + nd;
   const int ns = I.n_species;  // 1 or 2
-  const int i = (int)(nd / I.N2);
+  const int i = (int)nd / I.N2;  // (a grid's nodes fit 32 bits; 64-bit division is a long instruction sequence)
   const bool interior = i > 0 && i < I.n1;
   const bool extrap = I.guess && d.stp[inst].step >= 2;
   const Pop& P0 = d.pop[I.pop0];
@@ -62,7 +62,7 @@ __device__ __forceinline__ void grad_node(const DevPtrs& d, const Inst& I, long 
   const double* p = d.phi + I.node_off;
   const bool nofield = (I.flags & APIC_NO_FIELD) != 0;
   const int n1 = I.n1, n2 = I.n2, N2 = I.N2;
-  const int i = (int)(nd / N2), j = (int)(nd % N2);
+  const int i = (int)nd / N2, j = (int)nd - i * N2;
   double g1 = 0.0, g2 = 0.0;
   if (!nofield) {
     if (i == 0) g1 = (-3.0 * p[j] + 4.0 * p[N2 + j] - p[2 * N2 + j]) * I.i2h1;
