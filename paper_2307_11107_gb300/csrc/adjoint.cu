@@ -15,12 +15,12 @@
 //   push        per particle, the transpose of its local Jacobian (the step's
 //               gather of Eq. 10, Boris push of Eq. 9, chord, rotation and
 //               Eq. 2, or the tallies of an absorbed particle) applied to its
-//               adjoint; the local Jacobian comes from dual numbers, three
-//               directions at a time (state, gathered field, alpha, B);
+//               adjoint, stage by stage;
 //   surface     the seeds of the electric force and grain charge on phi;
 //   gradients   the transpose of the node differences;
 //   Poisson     lambda_b = A^-T lambda_phi with the nested-dissection fronts
-//               of A applied transposed (FP64), and the terms of phi_g (the
+//               of A applied transposed (FP64; as dataflow sweeps, nd_solve.cu,
+//               or, where a front exceeds their records, level by level), and the terms of phi_g (the
 //               Dirichlet row) and alpha (the operator's derivative);
 //   deposit     the transpose of the bilinear weighing onto the particles and
 //               the alpha-derivative of w = V_domain / N and of the volumes.
@@ -29,6 +29,7 @@
 // node-side kernels only in the double build (APIC_ADJOINT_COMMON).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "apic_internal.h"
@@ -45,16 +46,7 @@ namespace {
 #include "particle_common.cuh"
 
 using Real2 = typename Pair<Real>::T;
-template <int N>
-using DN = ad::Dual<Real, N>;
-using D3 = DN<3>;
-using D1 = DN<1>;
-
-__device__ __forceinline__ Real val(Real x) { return x; }
-template <int N>
-__device__ __forceinline__ Real val(const ad::Dual<Real, N>& x) {
-  return x.v;
-}
+using D1 = ad::Dual<Real, 1>;
 
 __device__ __forceinline__ const Real* ckc(const AdjPtrs& a, int k, int c) {
   return (const Real*)a.ck + ((long long)k * 5 + c) * a.stride;
@@ -73,76 +65,72 @@ __device__ __forceinline__ void pop_prefix_at(const DevPtrs& d, const PopState* 
   __syncthreads();
 }
 
-// One particle's push in number type T, the same sequence as the step's push
-// (gather of Eq. 10 with the bilinear weights of the cell the values give,
-// Boris push with the field vector -B z-hat, straight chord, rotation back to
-// the meridional plane, Eq. 2).  dg1, dg2 are added to the gathered node
-// gradients (zero: their directions carry the field's adjoint).
-template <class T>
+// What a population's particles share in the forward push, in their precision
+// (a conversion or a division of the FP64 parameters per particle bounds the
+// kernel: the FP64 pipe takes two lanes a clock per SM; 2e6 particles 70 us
+// with them, 49 without).
+struct FwdPop {
+  Real h, al, dt, B, h1, h2, x1_out;
+  long long base, node_off;
+  int n1, n2, N2, pad;
+};
+
+// One particle's push, the same sequence as the step's push (gather of Eq. 10
+// with the bilinear weights of its cell, Boris push with the field vector
+// -B z-hat, straight chord, rotation back to the meridional plane, Eq. 2).
 struct PushIO {
-  T x1n, x2n, vRn, vz, vTn;  // the new state of a kept particle
-  T R, Z, vx, vy;            // chord start and the velocity at n + 1/2 (tallies)
-  Real w[4];                 // gather weights (values) of the corners below
-  long long n[4];
+  Real x1n, x2n, vRn, vz, vTn;  // the new state of a kept particle
+  Real R, Z, vx, vy;            // chord start and the velocity at n + 1/2 (tallies)
   bool hit, out;
 };
 
-template <class T>
-__device__ __forceinline__ void push_eval(const Inst& I, const Real2* G, T x1, T x2, T vR, T vZ, T vT, T dg1, T dg2,
-                                          T al, T B, Real h, PushIO<T>& o) {
-  const Real dt = (Real)I.dt;
-  T r = radius(al, x1, x2);
-  T sn = sqrt((Real(1) - x2) * (Real(1) + x2));
-  T R = r * sn, Z = r * x2;
-  T u1 = (x1 + Real(1)) / (Real)I.h1;
-  T u2 = (x2 + Real(1)) / (Real)I.h2;
-  int ci = (int)floor(val(u1)), cj = (int)floor(val(u2));
-  ci = ci < 0 ? 0 : (ci > I.n1 - 1 ? I.n1 - 1 : ci);
-  cj = cj < 0 ? 0 : (cj > I.n2 - 1 ? I.n2 - 1 : cj);
-  T f1 = u1 - (Real)ci, f2 = u2 - (Real)cj;
-  if (val(f1) < Real(0)) f1 = T(Real(0));
-  if (val(f1) > Real(1)) f1 = T(Real(1));
-  if (val(f2) < Real(0)) f2 = T(Real(0));
-  if (val(f2) > Real(1)) f2 = T(Real(1));
-  const long long n00 = I.node_off + (long long)ci * I.N2 + cj;
-  o.n[0] = n00;
-  o.n[1] = n00 + I.N2;
-  o.n[2] = n00 + 1;
-  o.n[3] = n00 + I.N2 + 1;
-  const Real2 a00 = G[o.n[0]], a10 = G[o.n[1]], a01 = G[o.n[2]], a11 = G[o.n[3]];
-  T w00 = (Real(1) - f1) * (Real(1) - f2), w10 = f1 * (Real(1) - f2);
-  T w01 = (Real(1) - f1) * f2, w11 = f1 * f2;
-  o.w[0] = val(w00);
-  o.w[1] = val(w10);
-  o.w[2] = val(w01);
-  o.w[3] = val(w11);
-  T g1 = w00 * a00.x + w10 * a10.x + w01 * a01.x + w11 * a11.x + dg1;
-  T g2 = w00 * a00.y + w10 * a10.y + w01 * a01.y + w11 * a11.y + dg2;
-  Metric<T> m = metric(al, r, x2);
-  T ER = -(m.x1R * g1 + m.x2R * g2);
-  T EZ = -(m.x1Z * g1 + m.x2Z * g2);
-  T vx = vR + h * ER, vy = vT, vz = vZ + h * EZ;
-  T tz = h * (-B);
-  T sz = Real(2) * tz / (Real(1) + tz * tz);
-  T px_ = vx + vy * tz, py_ = vy - vx * tz;
+__device__ __forceinline__ void push_eval(const FwdPop& C, const Real2* G, Real x1, Real x2, Real vR, Real vZ, Real vT,
+                                          PushIO& o) {
+  const Real dt = C.dt, al = C.al, h = C.h;
+  Real r = radius(al, x1, x2);
+  Real sn = sqrt((Real(1) - x2) * (Real(1) + x2));
+  Real R = r * sn, Z = r * x2;
+  Real u1 = (x1 + Real(1)) / C.h1;
+  Real u2 = (x2 + Real(1)) / C.h2;
+  int ci = (int)floor(u1), cj = (int)floor(u2);
+  ci = ci < 0 ? 0 : (ci > C.n1 - 1 ? C.n1 - 1 : ci);
+  cj = cj < 0 ? 0 : (cj > C.n2 - 1 ? C.n2 - 1 : cj);
+  Real f1 = u1 - (Real)ci, f2 = u2 - (Real)cj;
+  if (f1 < Real(0)) f1 = Real(0);
+  if (f1 > Real(1)) f1 = Real(1);
+  if (f2 < Real(0)) f2 = Real(0);
+  if (f2 > Real(1)) f2 = Real(1);
+  const long long n00 = C.node_off + (long long)ci * C.N2 + cj;
+  const Real2 a00 = G[n00], a10 = G[n00 + C.N2], a01 = G[n00 + 1], a11 = G[n00 + C.N2 + 1];
+  Real w00 = (Real(1) - f1) * (Real(1) - f2), w10 = f1 * (Real(1) - f2);
+  Real w01 = (Real(1) - f1) * f2, w11 = f1 * f2;
+  Real g1 = w00 * a00.x + w10 * a10.x + w01 * a01.x + w11 * a11.x;
+  Real g2 = w00 * a00.y + w10 * a10.y + w01 * a01.y + w11 * a11.y;
+  Metric<Real> m = metric(al, r, x2);
+  Real ER = -(m.x1R * g1 + m.x2R * g2);
+  Real EZ = -(m.x1Z * g1 + m.x2Z * g2);
+  Real vx = vR + h * ER, vy = vT, vz = vZ + h * EZ;
+  Real tz = h * (-C.B);
+  Real sz = Real(2) * tz / (Real(1) + tz * tz);
+  Real px_ = vx + vy * tz, py_ = vy - vx * tz;
   vx = vx + py_ * sz;
   vy = vy - px_ * sz;
   vx = vx + h * ER;
   vz = vz + h * EZ;
-  T Xc = R + vx * dt, Yc = vy * dt, Zn = Z + vz * dt;
-  T Rn = sqrt(Xc * Xc + Yc * Yc);
-  T cr(Real(1)), sr(Real(0));
-  if (val(Rn) > Real(0)) {
+  Real Xc = R + vx * dt, Yc = vy * dt, Zn = Z + vz * dt;
+  Real Rn = sqrt(Xc * Xc + Yc * Yc);
+  Real cr(Real(1)), sr(Real(0));
+  if (Rn > Real(0)) {
     cr = Xc / Rn;
     sr = Yc / Rn;
   }
   o.vRn = cr * vx + sr * vy;
   o.vTn = -sr * vx + cr * vy;
-  T rn = sqrt(Rn * Rn + Zn * Zn);
+  Real rn = sqrt(Rn * Rn + Zn * Zn);
   o.x2n = Zn / rn;
-  o.hit = val(rn) < r_grain(val(al), val(o.x2n));
+  o.hit = rn < r_grain(al, o.x2n);
   o.x1n = x1_at(al, rn, o.x2n);
-  o.out = !o.hit && val(o.x1n) > (Real)I.x1_out;
+  o.out = !o.hit && o.x1n > C.x1_out;
   o.vz = vz;
   o.R = R;
   o.Z = Z;
@@ -151,10 +139,19 @@ __device__ __forceinline__ void push_eval(const Inst& I, const Real2* G, T x1, T
 }
 
 // ---- forward pass ----
-// The step's push (values), each slot's fate recorded: 0 kept, 1 absorbed,
-// 2 escaped, 3 no live particle.
+// The step's push (values), each live slot's state before it (the step's
+// checkpoint) and every slot's fate recorded: 0 kept, 1 absorbed, 2 escaped, 3
+// no live particle.
 __global__ void __launch_bounds__(256) k_adj_fwd_push(DevPtrs d, AdjPtrs a, int k) {
+  extern __shared__ __align__(16) char s_raw[];
+  FwdPop* s_pop = (FwdPop*)s_raw;
   __shared__ long long s_pre[kMaxPop + 1];
+  for (int p = threadIdx.x; p < d.n_pop; p += blockDim.x) {
+    const Pop& P = d.pop[p];
+    const Inst& I = d.inst[P.inst];
+    s_pop[p] = FwdPop{Real(0.5) * (Real)(P.q / P.m) * (Real)I.dt, (Real)I.alpha, (Real)I.dt, (Real)I.B, (Real)I.h1,
+                      (Real)I.h2, (Real)I.x1_out, P.base, I.node_off, I.n1, I.n2, I.N2, 0};
+  }
   pop_prefix_at(d, d.ps, s_pre);
   const long long total = s_pre[d.n_pop];
   const Real2* G = (const Real2*)d.G;
@@ -162,20 +159,27 @@ __global__ void __launch_bounds__(256) k_adj_fwd_push(DevPtrs d, AdjPtrs a, int 
   for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < total;
        q += (long long)gridDim.x * blockDim.x) {
     const int pop = find_pop(s_pre, d.n_pop, q);
-    const Pop& P = d.pop[pop];
-    const Inst& I = d.inst[P.inst];
-    const long long kk = q - s_pre[pop], slot = P.base + kk;
+    const FwdPop& C = s_pop[pop];
+    const long long kk = q - s_pre[pop], slot = C.base + kk;
     const Real x1 = ((const Real*)d.x1)[slot];
     if (!(x1 < Real(0))) {
       fate[slot] = 3;
       continue;
     }
-    PushIO<Real> o;
-    const Real h = Real(0.5) * (Real)(P.q / P.m) * (Real)I.dt;
-    push_eval<Real>(I, G, x1, ((const Real*)d.x2)[slot], ((const Real*)d.vR)[slot], ((const Real*)d.vZ)[slot],
-                    ((const Real*)d.vT)[slot], Real(0), Real(0), (Real)I.alpha, (Real)I.B, h, o);
+    const Real x2 = ((const Real*)d.x2)[slot], vR = ((const Real*)d.vR)[slot], vZ = ((const Real*)d.vZ)[slot],
+               vT = ((const Real*)d.vT)[slot];
+    Real* ck = (Real*)a.ck + (long long)k * 5 * a.stride + slot;
+    ck[0] = x1;
+    ck[a.stride] = x2;
+    ck[2 * a.stride] = vR;
+    ck[3 * a.stride] = vZ;
+    ck[4 * a.stride] = vT;
+    PushIO o;
+    push_eval(C, G, x1, x2, vR, vZ, vT, o);
     if (o.hit) {
-      absorb_tally(d, I, P, o.R, o.Z, o.vx, o.vz, o.vy, (Real)I.dt);
+      const Pop& P = d.pop[pop];
+      const Inst& I = d.inst[P.inst];
+      absorb_tally(d, I, P, o.R, o.Z, o.vx, o.vz, o.vy, C.dt);
       atomicAdd((unsigned long long*)&d.ps[pop].absorbed, 1ull);
       ((Real*)d.x1)[slot] = Real(2);
       push_hole(d, P, pop, kk);
@@ -185,7 +189,7 @@ __global__ void __launch_bounds__(256) k_adj_fwd_push(DevPtrs d, AdjPtrs a, int 
     if (o.out) {
       atomicAdd((unsigned long long*)&d.ps[pop].escaped, 1ull);
       ((Real*)d.x1)[slot] = Real(2);
-      push_hole(d, P, pop, kk);
+      push_hole(d, d.pop[pop], pop, kk);
       fate[slot] = 2;
       continue;
     }
@@ -197,6 +201,10 @@ __global__ void __launch_bounds__(256) k_adj_fwd_push(DevPtrs d, AdjPtrs a, int 
     fate[slot] = 0;
   }
 }
+
+// Threads per CTA of the injection kernels: a long chain of FP64 and special
+// functions for a few thousand particles, spread over the SMs.
+constexpr int kInjThreads = 64;
 
 // An injected particle's state (values and alpha-derivative) from its draws:
 // x2 from the inverse CDF of Eq. 4 on x1_out (its alpha-derivative from the
@@ -262,7 +270,7 @@ __device__ __forceinline__ void inject_eval(const DevPtrs& d, const TanPtrs& t, 
 
 // The step's surface injection (values), each draw's slot recorded (from the
 // population's base; -1 absorbed in its first flight, -2 escaped).
-__global__ void __launch_bounds__(256) k_adj_fwd_inject(DevPtrs d, AdjPtrs a, TanPtrs t, int k) {
+__global__ void __launch_bounds__(kInjThreads) k_adj_fwd_inject(DevPtrs d, AdjPtrs a, TanPtrs t, int k) {
   const int pop = blockIdx.y;
   const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   PopState& S = d.ps[pop];
@@ -331,7 +339,7 @@ __device__ __forceinline__ void add_grad(const AdjPtrs& a, int inst, double ga, 
 // (before the step's injection it held no particle, or one that left in
 // this step's push); a particle absorbed in its first flight adds its
 // tallies' alpha-derivatives (w = V_domain / N moves with alpha too).
-__global__ void __launch_bounds__(256) k_adj_rev_inject(DevPtrs d, AdjPtrs a, TanPtrs t, int k) {
+__global__ void __launch_bounds__(kInjThreads) k_adj_rev_inject(DevPtrs d, AdjPtrs a, TanPtrs t, int k) {
   const int pop = blockIdx.y;
   const Pop& P = d.pop[pop];
   const Inst& I = d.inst[P.inst];
@@ -368,139 +376,311 @@ __global__ void __launch_bounds__(256) k_adj_rev_inject(DevPtrs d, AdjPtrs a, Ta
   add_grad(a, inst, ga, 0.0, 0.0);
 }
 
+// A float as a double by integer arithmetic (exact; subnormals as zero): the
+// FP64 pipe, which a conversion instruction takes as long as a product, does
+// two lanes a clock per SM and bounds the reverse particle kernels.
+__device__ __forceinline__ double wide(double x) { return x; }
+__device__ __forceinline__ double wide(float x) {
+  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+  unsigned hi = (m >> 3) + 0x38000000u;
+  if (m >= 0x7f800000u) hi += 0x38000000u;  // infinities and NaN keep the largest exponent
+  if (m < 0x00800000u) hi = 0u;
+  return __hiloint2double((int)(hi | (b & 0x80000000u)), m < 0x00800000u ? 0 : (int)(b << 29));
+}
+
+// What a population's particles share in the reverse push.
+struct RevPop {
+  double c, s, dt;       // the magnetic rotation
+  double k0, k3, k2;     // the absorbed particle's seeds: dL/d(vz), dL/d(R vy) and its constant part
+  double dl;             // d ln w / d alpha
+  Real h, al, fdt, tz, sz, cB, sB;
+  Real h1, h2, ih1, ih2;
+  long long base, node_off;
+  int n1, n2, N2, inst;
+};
+
+// Cell and fractions of (x1, x2) as push_eval's, and the fractions' derivatives
+// (zero where the fraction is clamped).
+struct RevCell {
+  long long n00;
+  Real f1, f2, d1, d2;
+};
+__device__ __forceinline__ RevCell rev_cell(const RevPop& C, Real x1, Real x2) {
+  const Real u1 = (x1 + Real(1)) / C.h1, u2 = (x2 + Real(1)) / C.h2;
+  int ci = (int)floor(u1), cj = (int)floor(u2);
+  ci = ci < 0 ? 0 : (ci > C.n1 - 1 ? C.n1 - 1 : ci);
+  cj = cj < 0 ? 0 : (cj > C.n2 - 1 ? C.n2 - 1 : cj);
+  RevCell r{C.node_off + (long long)ci * C.N2 + cj, u1 - (Real)ci, u2 - (Real)cj, C.ih1, C.ih2};
+  if (r.f1 < Real(0) || r.f1 > Real(1)) {
+    r.f1 = r.f1 < Real(0) ? Real(0) : Real(1);
+    r.d1 = Real(0);
+  }
+  if (r.f2 < Real(0) || r.f2 > Real(1)) {
+    r.f2 = r.f2 < Real(0) ? Real(0) : Real(1);
+    r.d2 = Real(0);
+  }
+  return r;
+}
+
 // Push of step k backwards.  For each slot live at the start of the step
 // (the checkpoint), the transpose of the particle's local Jacobian applied to
 // the adjoint of its push's result: the new state's adjoint for a kept
 // particle, the output seeds of its tallies for an absorbed one, nothing for
-// an escaped one.  The local Jacobian comes from push_eval on three-direction
-// duals in three passes: (x1, x2, vR), (vZ, vTheta, g1), (g2, alpha, B).
-// The slot's adjoint becomes that of its state at the start of the step; the
-// gathered field's adjoint goes to the four corner nodes with the bilinear
-// weights.
-__global__ void __launch_bounds__(256) k_adj_rev_push(DevPtrs d, AdjPtrs a, TanPtrs t, int k) {
+// an escaped one.  The slot's adjoint becomes that of its state at the start
+// of the step; the gathered field's adjoint goes to the four corner nodes with
+// the bilinear weights.
+//
+// The push is taken backwards stage by stage (end point in Eq. 2, rotation to
+// the meridional plane, chord, Boris rotation, field and metric, Eq. 3), with
+// the stages' derivatives in closed form in the particles' precision and the
+// adjoints in FP64.  Bound: with float particles the FP64 pipe (about 45
+// products a particle and the corner sums), with double ones its operations
+// altogether.  Dual numbers three directions at a time, the form before,
+// evaluated the push's values three times and spent as much of the FP64 pipe
+// on converting the Jacobian's 45 entries as on their products.
+// The corner sums of a plasma that fills its volume meet on the outermost rows'
+// nodes, where the additions follow one another at L2 (its busiest slice at 87 %
+// while the mean is at 13 %): the CTAs add to several copies of lambda_G
+// (a.copies), folded before the gradients' transpose.  2e6 float particles on
+// 256 x 128 cells: 1.00 ms by duals, 0.48 in this form, 0.23 with eight copies.
+template <class F>
+__device__ __forceinline__ void load_pops(const DevPtrs& d, const AdjPtrs& a, const TanPtrs& t, F* pop) {
+  for (int p = threadIdx.x; p < d.n_pop; p += blockDim.x) {
+    const Pop& P = d.pop[p];
+    const Inst& I = d.inst[P.inst];
+    F& C = pop[p];
+    const double* sd = a.seed + (long long)P.inst * kNOut;
+    const double dt = I.dt, w = P.w;
+    C.h = Real(0.5) * (Real)(P.q / P.m) * (Real)I.dt;
+    C.al = (Real)I.alpha;
+    C.fdt = (Real)I.dt;
+    C.tz = C.h * -(Real)I.B;
+    const Real den = Real(1) + C.tz * C.tz;
+    C.sz = Real(2) * C.tz / den;
+    const Real cr = (Real(1) - C.tz * C.tz) / den;  // 1 - t s
+    C.c = cr;
+    C.s = C.sz;
+    // along B: dt = -h dB, ds = 2 c / (1 + t^2) dt, dc = -2 s / (1 + t^2) dt
+    C.sB = -C.h * (Real(2) * cr / den);
+    C.cB = C.h * (Real(2) * C.sz / den);
+    C.dt = (Real)I.dt;
+    C.dl = t.dlnw[P.inst];
+    C.k0 = sd[0] / dt * P.m * w;
+    C.k3 = sd[3] / dt * P.m * w;
+    C.k2 = sd[2] / dt * P.q * w;
+    C.h1 = (Real)I.h1;
+    C.h2 = (Real)I.h2;
+    C.ih1 = Real(1) / C.h1;
+    C.ih2 = Real(1) / C.h2;
+    C.base = P.base;
+    C.node_off = I.node_off;
+    C.n1 = I.n1;
+    C.n2 = I.n2;
+    C.N2 = I.N2;
+    C.inst = P.inst;
+  }
+  __syncthreads();
+}
+
+constexpr int kRevThreads = 256;
+__global__ void __launch_bounds__(kRevThreads) k_adj_rev_push(DevPtrs d, AdjPtrs a, TanPtrs t, int k) {
+  extern __shared__ __align__(16) char s_raw[];
+  RevPop* s_pop = (RevPop*)s_raw;
   __shared__ long long s_pre[kMaxPop + 1];
   const PopState* ps = a.ck_ps + (long long)k * d.n_pop;
+  load_pops(d, a, t, s_pop);
   pop_prefix_at(d, ps, s_pre);
   const long long total = s_pre[d.n_pop];
   const Real2* G = (const Real2*)a.Gk;
   const uint8_t* fate = a.fate + (long long)k * a.stride;
   const long long tn = d.total_nodes;
+  double* L = a.lam;
+  double* lG = a.lG + 2 * tn * (blockIdx.x % (unsigned)a.copies);
+  double ga = 0.0, gb = 0.0;
+  int inst = -1;  // the instance that ga, gb belong to
   for (long long q0 = (long long)blockIdx.x * blockDim.x; q0 < total; q0 += (long long)gridDim.x * blockDim.x) {
     const long long q = q0 + threadIdx.x;
-    double ga = 0.0, gb = 0.0;
-    int inst = -1;
-    if (q < total) {
-      const int pop = find_pop(s_pre, d.n_pop, q);
-      const Pop& P = d.pop[pop];
-      const Inst& I = d.inst[P.inst];
-      const long long slot = P.base + (q - s_pre[pop]);
-      const int f = fate[slot];
-      double* L = a.lam;
-      if (f == 0 || f == 1) {
-        inst = P.inst;
-        double lout[5];
-#pragma unroll
-        for (int c = 0; c < 5; ++c) lout[c] = f == 0 ? L[(long long)c * a.stride + slot] : 0.0;
-        const double* sd = a.seed + (long long)P.inst * kNOut;
-        const double dt = I.dt, w = P.w, dl = t.dlnw[P.inst];
-        const Real xs[5] = {ckc(a, k, 0)[slot], ckc(a, k, 1)[slot], ckc(a, k, 2)[slot], ckc(a, k, 3)[slot],
-                            ckc(a, k, 4)[slot]};
-        const Real h = Real(0.5) * (Real)(P.q / P.m) * (Real)I.dt;
-        double lin[9];
-        Real wts[4];
-        long long nodes[4];
-#pragma unroll 1
-        for (int pass = 0; pass < 3; ++pass) {
-          D3 in[9];
-#pragma unroll
-          for (int z = 0; z < 9; ++z) {
-            const Real v = z < 5 ? xs[z] : (z == 7 ? (Real)I.alpha : (z == 8 ? (Real)I.B : Real(0)));
-            in[z] = (z / 3 == pass) ? D3::seed(v, z % 3) : D3(v);
-          }
-          PushIO<D3> o;
-          push_eval<D3>(I, G, in[0], in[1], in[2], in[3], in[4], in[5], in[6], in[7], in[8], h, o);
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            wts[c] = o.w[c];
-            nodes[c] = o.n[c];
-          }
-#pragma unroll
-          for (int e = 0; e < 3; ++e) {
-            const int z = 3 * pass + e;
-            double acc;
-            if (f == 0) {
-              acc = lout[0] * (double)o.x1n.d[e] + lout[1] * (double)o.x2n.d[e] + lout[2] * (double)o.vRn.d[e] +
-                    lout[3] * (double)o.vz.d[e] + lout[4] * (double)o.vTn.d[e];
-            } else {
-              const double Rvy = (double)o.R.v * o.vy.v;
-              const double dRvy = (double)o.R.d[e] * o.vy.v + (double)o.R.v * o.vy.d[e];
-              const double a_w = z == 7 ? dl : 0.0;  // w moves with alpha
-              acc = sd[0] / dt * P.m * w * ((double)o.vz.d[e] + (double)o.vz.v * a_w) +
-                    sd[3] / dt * P.m * w * (dRvy + Rvy * a_w) + sd[2] / dt * P.q * w * a_w;
-            }
-            lin[z] = acc;
-          }
-        }
-#pragma unroll
-        for (int c = 0; c < 5; ++c) L[(long long)c * a.stride + slot] = lin[c];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          if (wts[c] == Real(0)) continue;
-          atomicAdd(a.lG + nodes[c], (double)wts[c] * lin[5]);
-          atomicAdd(a.lG + tn + nodes[c], (double)wts[c] * lin[6]);
-        }
-        ga = lin[7];
-        gb = lin[8];
-      } else {
-#pragma unroll
-        for (int c = 0; c < 5; ++c) L[(long long)c * a.stride + slot] = 0.0;
-      }
+    const int pop = q < total ? find_pop(s_pre, d.n_pop, q) : -1;
+    const int in_q = pop < 0 ? inst : s_pop[pop].inst;
+    if (__any_sync(0xffffffffu, in_q != inst)) {
+      add_grad(a, inst, ga, 0.0, gb);
+      ga = gb = 0.0;
+      inst = in_q;
     }
-    add_grad(a, inst, ga, 0.0, gb);
+    if (pop < 0) continue;
+    const RevPop& C = s_pop[pop];
+    const long long slot = C.base + (q - s_pre[pop]);
+    const int f = fate[slot];
+    if (f > 1) {
+#pragma unroll
+      for (int c = 0; c < 5; ++c) L[(long long)c * a.stride + slot] = 0.0;
+      continue;
+    }
+    const Real x1 = ckc(a, k, 0)[slot], x2 = ckc(a, k, 1)[slot], vR = ckc(a, k, 2)[slot], vZ = ckc(a, k, 3)[slot],
+               vT = ckc(a, k, 4)[slot];
+    const Real al = C.al, h = C.h, dt = C.fdt;
+    // Eq. 3 and the position: derivatives along x1, x2, alpha
+    const Real qs = sqrt(Real(1) - Real(4) * al * x1 * x2), iq = Real(1) / qs, ix = Real(1) / x1;
+    const Real r = -(Real(1) + qs) * (Real(0.5) * ix), ir = Real(1) / r;
+    const Real s2 = (Real(1) - x2) * (Real(1) + x2), sn = sqrt(s2);
+    const Real sn2 = sn > Real(0) ? -x2 / sn : Real(0);
+    const Real r1 = (al * x2 * iq - r) * ix, r2 = al * iq, ra = x2 * iq;
+    const Real R = r * sn, Z = r * x2;
+    const Real R1 = r1 * sn, R2 = r2 * sn + r * sn2, Ra = ra * sn;
+    const Real Z1 = r1 * x2, Z2 = r2 * x2 + r, Za = ra * x2;
+    // the field of Eq. 10 and its derivatives
+    const RevCell e = rev_cell(C, x1, x2);
+    const Real2 a00 = G[e.n00], a10 = G[e.n00 + C.N2], a01 = G[e.n00 + 1], a11 = G[e.n00 + C.N2 + 1];
+    const Real o1 = Real(1) - e.f1, o2 = Real(1) - e.f2;
+    const Real w00 = o1 * o2, w10 = e.f1 * o2, w01 = o1 * e.f2, w11 = e.f1 * e.f2;
+    const Real g1 = w00 * a00.x + w10 * a10.x + w01 * a01.x + w11 * a11.x;
+    const Real g2 = w00 * a00.y + w10 * a10.y + w01 * a01.y + w11 * a11.y;
+    const Real g11 = e.d1 * (o2 * (a10.x - a00.x) + e.f2 * (a11.x - a01.x));
+    const Real g12 = e.d2 * (o1 * (a01.x - a00.x) + e.f1 * (a11.x - a10.x));
+    const Real g21 = e.d1 * (o2 * (a10.y - a00.y) + e.f2 * (a11.y - a01.y));
+    const Real g22 = e.d2 * (o1 * (a01.y - a00.y) + e.f1 * (a11.y - a10.y));
+    // the metric (geom.cuh) and its derivatives along r, x2, alpha
+    const Real ir3 = ir * ir * ir;
+    const Real p1 = r + Real(3) * al * x2, p2 = Real(3) * x2 * x2 - Real(1);
+    const Real mR1 = sn * p1 * ir3, mZ1 = (r * x2 + al * p2) * ir3, mR2 = -x2 * sn * ir, mZ2 = s2 * ir;
+    const Real mR1r = sn * ir3 - Real(3) * mR1 * ir, mZ1r = x2 * ir3 - Real(3) * mZ1 * ir;
+    const Real mR1x = (sn2 * p1 + Real(3) * al * sn) * ir3, mZ1x = (r + Real(6) * al * x2) * ir3;
+    const Real mR2x = -(sn + x2 * sn2) * ir, mZ2x = Real(-2) * x2 * ir;
+    const Real ER = -(mR1 * g1 + mR2 * g2), EZ = -(mZ1 * g1 + mZ2 * g2);
+    const Real ERr = -(mR1r * g1 - mR2 * ir * g2), EZr = -(mZ1r * g1 - mZ2 * ir * g2);
+    const Real ER1 = ERr * r1 - (mR1 * g11 + mR2 * g21), EZ1 = EZr * r1 - (mZ1 * g11 + mZ2 * g21);
+    const Real ER2 = ERr * r2 - (mR1x * g1 + mR2x * g2 + mR1 * g12 + mR2 * g22);
+    const Real EZ2 = EZr * r2 - (mZ1x * g1 + mZ2x * g2 + mZ1 * g12 + mZ2 * g22);
+    const Real ERa = ERr * ra - Real(3) * sn * x2 * ir3 * g1, EZa = EZr * ra - p2 * ir3 * g1;
+    // Boris push
+    const Real bx = vR + h * ER, bz = vZ + h * EZ;
+    const Real px = bx + vT * C.tz, py = vT - bx * C.tz;
+    const Real vx = bx + py * C.sz + h * ER, vy = vT - px * C.sz, vz = bz + h * EZ;
+    double aX = 0.0, aY = 0.0, aZ = 0.0;     // of the chord's end
+    double avx = 0.0, avy = 0.0, avz, aR = 0.0, aa = 0.0;
+    if (f == 0) {
+      const double l1 = L[slot], l2 = L[a.stride + slot], lR = L[2 * a.stride + slot], lZ = L[3 * a.stride + slot],
+                   lT = L[4 * a.stride + slot];
+      const Real Xc = R + vx * dt, Yc = vy * dt, Zn = Z + vz * dt;
+      const Real Rn = sqrt(Xc * Xc + Yc * Yc), rn = sqrt(Rn * Rn + Zn * Zn), irn = Real(1) / rn;
+      Real cr = Real(1), sr = Real(0), iRn = Real(0);
+      if (Rn > Real(0)) {
+        iRn = Real(1) / Rn;
+        cr = Xc * iRn;
+        sr = Yc * iRn;
+      }
+      const Real xn = Zn * irn, st = Rn * irn, i2 = irn * irn;
+      // Eq. 2, then x2 = Z / r and r of the end point
+      aa = l1 * wide(-xn * i2);
+      const double ax2 = fma(l1, wide(-al * i2), l2);
+      const double arn = l1 * wide(i2 + Real(2) * al * xn * i2 * irn);
+      aZ = fma(arn, wide(xn), ax2 * wide(st * st * irn));
+      const double aRn = iRn > Real(0) ? wide(st) * fma(ax2, wide(-xn * irn), arn) : 0.0;
+      // rotation to the meridional plane
+      const Real vRn = cr * vx + sr * vy, vTn = cr * vy - sr * vx;
+      const double tt = fma(lR, wide(vTn), -(lT * wide(vRn)));
+      aX = fma(aRn, wide(cr), tt * wide(-sr * iRn));
+      aY = fma(aRn, wide(sr), tt * wide(cr * iRn));
+      const double c = wide(cr), s = wide(sr);
+      avx = fma(C.dt, aX, fma(lR, c, -(lT * s)));
+      avy = fma(C.dt, aY, fma(lR, s, lT * c));
+      avz = fma(C.dt, aZ, lZ);
+      aR = aX;
+    } else {
+      const double Rw = wide(R), vyw = wide(vy);
+      avz = C.k0;
+      aR = C.k3 * vyw;
+      avy = C.k3 * Rw;
+      aa = C.dl * (C.k0 * wide(vz) + C.k3 * Rw * vyw + C.k2);  // w moves with alpha
+    }
+    // Boris rotation: vx = c bx + s vT + h ER, vy = c vT - s bx
+    gb += avx * wide(bx * C.cB + vT * C.sB) + avy * wide(vT * C.cB - bx * C.sB);
+    const double abx = fma(C.c, avx, -(C.s * avy)), aT = fma(C.s, avx, C.c * avy);
+    const double aE = avx + abx;  // over h; that of h EZ is 2 avz
+    const Real hz = Real(2) * h;
+    const double l1 = fma(aR, wide(R1), fma(aZ, wide(Z1), fma(aE, wide(h * ER1), avz * wide(hz * EZ1))));
+    const double l2 = fma(aR, wide(R2), fma(aZ, wide(Z2), fma(aE, wide(h * ER2), avz * wide(hz * EZ2))));
+    ga += aa + fma(aR, wide(Ra), fma(aZ, wide(Za), fma(aE, wide(h * ERa), avz * wide(hz * EZa))));
+    const double lg1 = -fma(aE, wide(h * mR1), avz * wide(hz * mZ1));
+    const double lg2 = -fma(aE, wide(h * mR2), avz * wide(hz * mZ2));
+    L[slot] = l1;
+    L[a.stride + slot] = l2;
+    L[2 * a.stride + slot] = abx;
+    L[3 * a.stride + slot] = avz;
+    L[4 * a.stride + slot] = aT;
+    const Real w[4] = {w00, w10, w01, w11};
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      if (w[c] == Real(0)) continue;
+      const long long n = e.n00 + (c & 1 ? C.N2 : 0) + (c >> 1);
+      const double wd = wide(w[c]);
+      atomicAdd(lG + n, wd * lg1);
+      atomicAdd(lG + tn + n, wd * lg2);
+    }
   }
+  add_grad(a, inst, ga, 0.0, gb);
 }
 
 // Deposit of step k backwards: rho = sum_p q w S(x_p) / V, so the adjoint of
 // a live particle's (x1, x2) gains q w sum_c (dS_c / dx) lambda_rho_c / V_c
-// (bilinear weights of its cell; a clamped fraction carries none).
-__global__ void __launch_bounds__(256) k_adj_rev_deposit(DevPtrs d, AdjPtrs a, int k) {
+// (bilinear weights of its cell; a clamped fraction carries none; a.lrho holds
+// lambda_rho / V).  Bound by the FP64 pipe: a coordinate's cell and fraction
+// come from one fused product and a conversion (as in cell_fixed.cuh), the
+// corner sum from the cell's differences.
+// 2e6 float particles on 256 x 128 cells: 475 us with divisions, 63 so.
+struct DepPop {
+  double s1, s2;            // 2^b / h1, 2^b / h2
+  double k1, k2;            // q w / h1, q w / h2
+  long long base, node_off;
+  int n1, n2, N2, b;        // b: a fraction's bits (the largest cell index and a fraction share 62)
+};
+
+// Cell of a logical coordinate and the fraction in it (to 2^-b); the
+// fraction's derivative is zero (d = 0) where it is clamped to [0, 1].
+__device__ __forceinline__ int dep_cell(double x, double s, int n, int b, double& f, double& d) {
+  const long long t = __double2ll_rn(fma(x, s, s));
+  const int i = (int)(t >> b);
+  unsigned long long m = (unsigned long long)t & ((1ull << b) - 1ull);
+  if ((unsigned)i >= (unsigned)n) {  // outside the grid, or on its last node
+    m = i < 0 ? 0ull : 1ull << b;
+    if (t != (long long)n << b) d = 0.0;
+  }
+  f = __longlong_as_double((long long)(0x3ff0000000000000ull + (m << (52 - b)))) - 1.0;
+  return min(max(i, 0), n - 1);
+}
+
+__global__ void __launch_bounds__(kRevThreads) k_adj_rev_deposit(DevPtrs d, AdjPtrs a, int k) {
+  extern __shared__ __align__(16) char s_raw[];
+  DepPop* s_pop = (DepPop*)s_raw;
   __shared__ long long s_pre[kMaxPop + 1];
-  const PopState* ps = a.ck_ps + (long long)k * d.n_pop;
-  pop_prefix_at(d, ps, s_pre);
+  for (int p = threadIdx.x; p < d.n_pop; p += blockDim.x) {
+    const Pop& P = d.pop[p];
+    const Inst& I = d.inst[P.inst];
+    const double qw = P.q * P.w;
+    int b = 50;
+    while (b > 1 && (long long)max(I.n1, I.n2) >> (62 - b)) --b;
+    s_pop[p] = DepPop{ldexp(1.0 / I.h1, b), ldexp(1.0 / I.h2, b), qw / I.h1, qw / I.h2, P.base, I.node_off, I.n1, I.n2,
+                      I.N2, b};
+  }
+  pop_prefix_at(d, a.ck_ps + (long long)k * d.n_pop, s_pre);
   const long long total = s_pre[d.n_pop];
   const uint8_t* fate = a.fate + (long long)k * a.stride;
   for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < total;
        q += (long long)gridDim.x * blockDim.x) {
     const int pop = find_pop(s_pre, d.n_pop, q);
-    const Pop& P = d.pop[pop];
-    const Inst& I = d.inst[P.inst];
-    const long long slot = P.base + (q - s_pre[pop]);
+    const DepPop& C = s_pop[pop];
+    const long long slot = C.base + (q - s_pre[pop]);
     if (fate[slot] == 3) continue;
-    const double x1 = (double)ckc(a, k, 0)[slot], x2 = (double)ckc(a, k, 1)[slot];
-    const double u1 = (x1 + 1.0) / I.h1, u2 = (x2 + 1.0) / I.h2;
-    int ci = (int)floor(u1), cj = (int)floor(u2);
-    ci = ci < 0 ? 0 : (ci > I.n1 - 1 ? I.n1 - 1 : ci);
-    cj = cj < 0 ? 0 : (cj > I.n2 - 1 ? I.n2 - 1 : cj);
-    double f1 = u1 - ci, f2 = u2 - cj, d1 = 1.0 / I.h1, d2 = 1.0 / I.h2;
-    if (f1 < 0.0 || f1 > 1.0) {
-      f1 = f1 < 0.0 ? 0.0 : 1.0;
-      d1 = 0.0;
-    }
-    if (f2 < 0.0 || f2 > 1.0) {
-      f2 = f2 < 0.0 ? 0.0 : 1.0;
-      d2 = 0.0;
-    }
-    const long long n00 = I.node_off + (long long)ci * I.N2 + cj;
-    const long long nn[4] = {n00, n00 + I.N2, n00 + 1, n00 + I.N2 + 1};
-    double l[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) l[c] = a.lrho[nn[c]] / d.V[nn[c]];
-    // dS/dx1 = d1 (-(1 - f2), (1 - f2), -f2, f2); dS/dx2 = d2 (-(1 - f1), -f1, (1 - f1), f1)
-    const double qw = P.q * P.w;
-    const double gx1 = d1 * (-(1.0 - f2) * l[0] + (1.0 - f2) * l[1] - f2 * l[2] + f2 * l[3]);
-    const double gx2 = d2 * (-(1.0 - f1) * l[0] - f1 * l[1] + (1.0 - f1) * l[2] + f1 * l[3]);
-    a.lam[slot] += qw * gx1;
-    a.lam[a.stride + slot] += qw * gx2;
+    double f1, f2, k1 = C.k1, k2 = C.k2;
+    const int ci = dep_cell(wide(ckc(a, k, 0)[slot]), C.s1, C.n1, C.b, f1, k1);
+    const int cj = dep_cell(wide(ckc(a, k, 1)[slot]), C.s2, C.n2, C.b, f2, k2);
+    const double* l = a.lrho + C.node_off + (long long)ci * C.N2 + cj;
+    // l00 .. l11 = l[0], l[N2], l[1], l[N2 + 1]:  d/dx1 = (l10 - l00) + f2 m, d/dx2 = (l01 - l00) + f1 m,
+    // m = (l11 - l01) - (l10 - l00)
+    const double l00 = l[0], l10 = l[C.N2], l01 = l[1], l11 = l[C.N2 + 1];
+    const double e1 = l10 - l00, e2 = l01 - l00, m = (l11 - l01) - e1;
+    a.lam[slot] = fma(k1, fma(f2, m, e1), a.lam[slot]);
+    a.lam[a.stride + slot] = fma(k2, fma(f1, m, e2), a.lam[a.stride + slot]);
   }
 }
 
@@ -521,52 +701,48 @@ __device__ double block_sum(double v, double* sh) {
   return r;
 }
 
-// Window sums of the step's outputs (before the step's bookkeeping clears the
-// step tallies).
-__global__ void k_adj_values(DevPtrs d, AdjPtrs a) {
-  const int inst = blockIdx.x * blockDim.x + threadIdx.x;
-  if (inst >= d.n_inst) return;
-  const Inst& I = d.inst[inst];
-  const StepState& T = d.stp[inst];
-  double tl[5];
-  step_tallies(d, inst, tl);
-  double* v = a.vals + (long long)inst * kNOut;
-  v[0] += tl[1] / I.dt;
-  v[1] += T.FZ;
-  v[2] += tl[0] / I.dt;
-  v[3] += tl[2] / I.dt;
-  v[4] += T.Q;
+// Constants of the grain surface per node j of instance blockIdx.x, and their
+// alpha-derivatives: |grad x1|, dA of Eq. 4 and n_Z dA (once, at set-up).
+__global__ void __launch_bounds__(256) k_adj_surface_geom(DevPtrs d, AdjPtrs a, int n2_max) {
+  const Inst& I = d.inst[blockIdx.x];
+  double* o = a.sgeo + 6ll * blockIdx.x * (n2_max + 1);
+  for (int j = threadIdx.x; j <= I.n2; j += blockDim.x) {
+    using DD = ad::Dual<double, 1>;
+    DD al = DD::seed(I.alpha, 0), X2(x2_node(I, j));
+    DD r = r_grain(al, X2);
+    Metric<DD> m = metric(al, r, X2);
+    DD g = sqrt(m.x1R * m.x1R + m.x1Z * m.x1Z);
+    DD dA = area_density(al, DD(-1.0), X2);
+    DD nzda = (m.x1Z / g) * dA;
+    const double v[6] = {g.v, g.d[0], dA.v, dA.d[0], nzda.v, nzda.d[0]};
+    for (int c = 0; c < 6; ++c) o[6 * j + c] = v[c];
+  }
 }
 
 // Seeds of the electric force and grain charge of step k on phi (rows 0..2
 // through the one-sided dphi/dx1 on the grain), and their alpha-derivative at
 // fixed phi (|grad x1|, n_Z and dA of Eq. 4 on the grain).
-__global__ void __launch_bounds__(256) k_adj_surface(DevPtrs d, AdjPtrs a, TanPtrs t, int k) {
+__global__ void __launch_bounds__(256) k_adj_surface(DevPtrs d, AdjPtrs a, int k, int n2_max) {
   __shared__ double sh[256];
   const int inst = blockIdx.x;
   const Inst& I = d.inst[inst];
   const bool nofield = (I.flags & APIC_NO_FIELD) != 0;
   const int N2 = I.N2;
   const double* p0 = a.ck_phi + (long long)k * d.total_nodes + I.node_off;
+  const double* geo = a.sgeo + 6ll * inst * (n2_max + 1);
   const double sF = a.seed[(long long)inst * kNOut + 1], sQ = a.seed[(long long)inst * kNOut + 4];
   double ga = 0.0;
   for (int j = threadIdx.x; j <= I.n2 && !nofield; j += blockDim.x) {
-    using DD = ad::Dual<double, 1>;
-    const double x2 = x2_node(I, j);
-    DD al = DD::seed(I.alpha, 0), X2(x2);
-    DD r = r_grain(al, X2);
-    Metric<DD> m = metric(al, r, X2);
-    DD g = sqrt(m.x1R * m.x1R + m.x1Z * m.x1Z);
-    DD dA = area_density(al, DD(-1.0), X2);
-    DD nzda = (m.x1Z / g) * dA;
+    const double g = geo[6 * j], gd = geo[6 * j + 1], dA = geo[6 * j + 2], dAd = geo[6 * j + 3], nz = geo[6 * j + 4],
+                 nzd = geo[6 * j + 5];
     const double G1 = (-3.0 * p0[j] + 4.0 * p0[N2 + j] - p0[2 * N2 + j]) / (2.0 * I.h1);
-    const double En = -G1 * g.v;
+    const double En = -G1 * g;
     const double tw = (j == 0 || j == I.n2) ? 0.5 * I.h2 : I.h2;
     // dL/dE_n and the E_n derivative along alpha at fixed phi
-    const double dLdE = sQ * tw * dA.v + sF * tw * En * nzda.v;
-    const double dEa = -G1 * g.d[0];
-    ga += dLdE * dEa + sQ * tw * En * dA.d[0] + sF * tw * 0.5 * En * En * nzda.d[0];
-    const double c = -g.v / (2.0 * I.h1);  // dE_n / dphi = c (-3, 4, -1) on rows 0, 1, 2
+    const double dLdE = sQ * tw * dA + sF * tw * En * nz;
+    const double dEa = -G1 * gd;
+    ga += dLdE * dEa + sQ * tw * En * dAd + sF * tw * 0.5 * En * En * nzd;
+    const double c = -g / (2.0 * I.h1);  // dE_n / dphi = c (-3, 4, -1) on rows 0, 1, 2
     double* lp = a.lphi + I.node_off;
     lp[j] += dLdE * c * -3.0;
     lp[N2 + j] += dLdE * c * 4.0;
@@ -574,6 +750,16 @@ __global__ void __launch_bounds__(256) k_adj_surface(DevPtrs d, AdjPtrs a, TanPt
   }
   const double tot = block_sum(ga, sh);
   if (threadIdx.x == 0 && tot != 0.0) atomicAdd(a.grad + (long long)inst * kNPar + 0, tot);
+}
+
+// The copies of lambda_G added into the first.
+__global__ void __launch_bounds__(256) k_adj_fold(double* lG, long long n, int copies) {
+  for (long long z = (long long)blockIdx.x * blockDim.x + threadIdx.x; z < n; z += (long long)gridDim.x * blockDim.x) {
+    double s = lG[z];
+#pragma unroll 4
+    for (int c = 1; c < copies; ++c) s += lG[c * n + z];
+    lG[z] = s;
+  }
 }
 
 // lambda_phi += D^T lambda_G: the transpose of the node gradients (central
@@ -691,7 +877,7 @@ __global__ void __launch_bounds__(256) k_adj_after_solve(DevPtrs d, AdjPtrs a, T
       ga -= lb * d.rscale[g] * dL;
       lr = -d.rscale[g] * lb;
     }
-    a.lrho[g] = lr;
+    a.lrho[g] = lr / d.V[g];  // as the deposit's weighing takes it
     ga += lr * rho[nd] * (dl - t.dV[g] / d.V[g]);
   }
   const double ta = block_sum(ga, sh), tp = block_sum(gp, sh);
@@ -704,42 +890,53 @@ __global__ void __launch_bounds__(256) k_adj_after_solve(DevPtrs d, AdjPtrs a, T
 
 }  // namespace
 
+// CTAs of 256 threads over `n` nodes.
+[[maybe_unused]] static unsigned node_blocks(long long n) {
+  return (unsigned)std::max<long long>(1, std::min<long long>(608, (n + 255) / 256));
+}
+
+// CTAs of 256 threads over every slot.
+static unsigned adj_blocks(const AdjPtrs& a) {
+  return (unsigned)std::max<long long>(1, std::min<long long>(kAdjBlocks, (a.stride + 255) / 256));
+}
+
 template <>
 void launch_adj_fwd_push<Real>(const DevPtrs& d, const AdjPtrs& a, int k, cudaStream_t s) {
-  k_adj_fwd_push<<<kAdjBlocks * 4, 256, 0, s>>>(d, a, k);
+  k_adj_fwd_push<<<adj_blocks(a), 256, sizeof(FwdPop) * (size_t)d.n_pop, s>>>(d, a, k);
 }
 template <>
 void launch_adj_fwd_inject<Real>(const DevPtrs& d, const AdjPtrs& a, const TanPtrs& t, int k, long long max_inj,
                                  cudaStream_t s) {
   if (max_inj <= 0) return;
-  const unsigned gx = (unsigned)((max_inj + 255) / 256);
-  k_adj_fwd_inject<<<dim3(gx, d.n_pop), 256, 0, s>>>(d, a, t, k);
+  const unsigned gx = (unsigned)((max_inj + kInjThreads - 1) / kInjThreads);
+  k_adj_fwd_inject<<<dim3(gx, d.n_pop), kInjThreads, 0, s>>>(d, a, t, k);
 }
 template <>
 void launch_adj_rev_inject<Real>(const DevPtrs& d, const AdjPtrs& a, const TanPtrs& t, int k, long long max_inj,
                                  cudaStream_t s) {
   if (max_inj <= 0) return;
-  const unsigned gx = (unsigned)((max_inj + 255) / 256);
-  k_adj_rev_inject<<<dim3(gx, d.n_pop), 256, 0, s>>>(d, a, t, k);
+  const unsigned gx = (unsigned)((max_inj + kInjThreads - 1) / kInjThreads);
+  k_adj_rev_inject<<<dim3(gx, d.n_pop), kInjThreads, 0, s>>>(d, a, t, k);
 }
 template <>
 void launch_adj_rev_push<Real>(const DevPtrs& d, const AdjPtrs& a, const TanPtrs& t, int k, cudaStream_t s) {
-  k_adj_rev_push<<<kAdjBlocks, 256, 0, s>>>(d, a, t, k);
+  k_adj_rev_push<<<adj_blocks(a), kRevThreads, sizeof(RevPop) * (size_t)d.n_pop, s>>>(d, a, t, k);
 }
 template <>
 void launch_adj_rev_deposit<Real>(const DevPtrs& d, const AdjPtrs& a, int k, cudaStream_t s) {
-  k_adj_rev_deposit<<<kAdjBlocks, 256, 0, s>>>(d, a, k);
+  k_adj_rev_deposit<<<adj_blocks(a), kRevThreads, sizeof(DepPop) * (size_t)d.n_pop, s>>>(d, a, k);
 }
 
 #ifdef APIC_ADJOINT_COMMON
-void launch_adj_values(const DevPtrs& d, const AdjPtrs& a, cudaStream_t s) {
-  k_adj_values<<<(d.n_inst + 63) / 64, 64, 0, s>>>(d, a);
+void launch_adj_surface_geom(const DevPtrs& d, const AdjPtrs& a, int n2_max, cudaStream_t s) {
+  k_adj_surface_geom<<<d.n_inst, 256, 0, s>>>(d, a, n2_max);
 }
-void launch_adj_surface(const DevPtrs& d, const AdjPtrs& a, const TanPtrs& t, int k, cudaStream_t s) {
-  k_adj_surface<<<d.n_inst, 256, 0, s>>>(d, a, t, k);
+void launch_adj_surface(const DevPtrs& d, const AdjPtrs& a, int k, int n2_max, cudaStream_t s) {
+  k_adj_surface<<<d.n_inst, 256, 0, s>>>(d, a, k, n2_max);
 }
 void launch_adj_gradT(const DevPtrs& d, const AdjPtrs& a, cudaStream_t s) {
-  k_adj_gradT<<<dim3(kRedBlocks, d.n_inst), 256, 0, s>>>(d, a);
+  if (a.copies > 1) k_adj_fold<<<node_blocks(2 * d.total_nodes), 256, 0, s>>>(a.lG, 2 * d.total_nodes, a.copies);
+  k_adj_gradT<<<dim3(node_blocks(d.total_nodes / d.n_inst), d.n_inst), 256, 0, s>>>(d, a);
 }
 void launch_adj_to_unknowns(const DevPtrs& d, const AdjPtrs& a, cudaStream_t s) {
   k_adj_to_unknowns<<<dim3(kRedBlocks, d.n_inst), 256, 0, s>>>(d, a);
@@ -749,7 +946,7 @@ void launch_adj_ndT(const AdjPtrs& a, int f0, int f1, long long unk0, int smem_d
   k_adj_ndT<<<f1 - f0, 256, sizeof(double) * (size_t)smem_doubles, s>>>(a, f0, unk0, forward ? 1 : 0);
 }
 void launch_adj_after_solve(const DevPtrs& d, const AdjPtrs& a, const TanPtrs& t, int k, cudaStream_t s) {
-  k_adj_after_solve<<<dim3(kRedBlocks, d.n_inst), 256, 0, s>>>(d, a, t, k);
+  k_adj_after_solve<<<dim3(node_blocks(d.total_nodes / d.n_inst), d.n_inst), 256, 0, s>>>(d, a, t, k);
 }
 const void* adj_ndT_kernel() { return (const void*)k_adj_ndT; }
 #endif

@@ -190,8 +190,13 @@ struct apic_sim {
   int win_rows = 0;                   // push deposit window rows (0: default for the grid), set by apic_autotune
   int chunk_group = 0;                // push chunks per group (0: default), set by apic_autotune
   int chunk_items = 0;                // vector push particles per thread of a chunk (0: default), apic_autotune
+  unsigned long long* dep_part = nullptr;  // the windows' copies of the deposit's accumulator
+  int dep_copies = 1;
   AdjPtrs adj{};                      // reverse-sweep state (allocated on first use, for up to adj_K steps)
   int adj_K = 0;
+  BcrPlan adj_plan{};                 // its transposed solve as dataflow sweeps (adj_blocks CTAs; 0: level by level)
+  DevPtrs adj_view{};                 // (their records and vectors alone)
+  int adj_blocks = 0;
   std::vector<std::vector<std::pair<int, int>>> adj_levels;  // per instance, per tree level: fronts [f0, f1)
   std::vector<int> adj_smem;                                  // per instance: doubles of a front's vector
 
@@ -620,6 +625,30 @@ void parallel_for(int n, F f) {
   for (auto& x : th) x.join();
 }
 
+// Instance k's records of a plan, from its fronts in Real, written and copied
+// to the batch's at `dst` (host copy of one instance at a time).
+template <class Real>
+bool upload_records(apic_sim* S, const NdFlowPlan& P, int k, const NdFlowInst& I, const NdFactor& f, int32_t* dst) {
+  std::vector<int32_t> rec((size_t)(P.words[k + 1] - P.words[k]));
+  size_t t0 = 0, t1;
+  while (t0 < P.tasks.size() && P.tasks[t0].inst < k) ++t0;
+  for (t1 = t0; t1 < P.tasks.size() && P.tasks[t1].inst == k;) ++t1;
+  const int n = (int)std::min<size_t>(64, t1 - t0);
+  parallel_for(n, [&](int q) {
+    for (size_t t = t0 + q; t < t1; t += n) {
+      int32_t* out = rec.data() + (P.off[t] - P.words[k]);
+      if constexpr (sizeof(Real) == 8)
+        nd_flow_write<double>(P.up, P.tasks[t], P.place, P.perm.data() + I.foff, I, f.fm64.data(), 0, f.nb64.data(),
+                              f.fm_total, out);
+      else
+        nd_flow_write<float>(P.up, P.tasks[t], P.place, P.perm.data() + I.foff, I, f.fm.data(), 0, f.nb.data(),
+                             f.fm_total, out);
+    }
+  });
+  S->h2d(dst + P.words[k], rec.data(), rec.size());
+  return S->sync();  // (the host copy goes)
+}
+
 double nd_coef(const void* ctx, int i, int j, int slot) { return ((const HostLevel*)ctx)->get(slot, i, j); }
 
 // Layout of instance I's reduction: block size, levels before the dense
@@ -975,10 +1004,7 @@ static int setup(apic_sim* S) {
   std::vector<NdFactor> nds(ni);
   std::vector<char> use_nd(ni, 0);
   NdUpload ndu;
-  std::vector<NdFlowTask> nd_tasks;   // the dataflow sweeps' records ...
-  std::vector<int64_t> nd_off;        // ... and their first words (of all instances' records)
-  std::vector<int32_t> nd_place, nd_perm;  // a front's first place among its instance's unknowns, an unknown's place
-  std::vector<int4> nd_list;          // the sweeps' record lists
+  NdFlowPlan fp;       // the dataflow sweeps' records
   long long nd_w = 0;  // elements of one right-hand side's update vectors
   constexpr int kElem = (int)(sizeof(Real) / sizeof(float));  // words per element of a dataflow solve's fronts
   {
@@ -1035,76 +1061,43 @@ static int setup(apic_sim* S) {
       double nodes = 0.0;
       for (int k = 0; k < ni; ++k) nodes += (double)S->inst[k].nodes;
       bcr_in.assign(ni, BcrInst{});
-      std::vector<int64_t> words(ni + 1, 0);  // first word of each instance's records
       for (int k = 0; k < ni && flow; ++k) {
         const Inst& I = S->inst[k];
         BcrInst& B = bcr_in[k];
-        NdLevels lvl;
-        const int f0 = (int)ndu.fronts.size();
-        nd_layout(nds[k], 0, nd_w, kNdWarpMaxS, kNdWarpMaxU, kNdWarpStage, kNdTaskFloats, kNdTaskRows, kNdTaskFronts,
-                  kNdUnitStage, 1, ndu, lvl);
-        const int nf = (int)ndu.fronts.size() - f0;
         // the share of the CTAs by nodes (the sums do not depend on the tasks)
         const int ctas = std::max(1, (int)std::lround(sms * (double)I.nodes / nodes));
-        const size_t t0 = nd_tasks.size();
-        for (int sw = 0; sw < 2 && flow; ++sw)
-          flow = nd_flow_tasks(ndu, f0, nf, nds[k].depth, k, sw == 0, kElem, nd_workers(kElem) * ctas, nd_vec_cap(kElem),
-                               kElem == 1 ? 4 * kNdUnits * ctas : 1 << 30, nd_tasks);
-        words[k + 1] = words[k];
-        for (size_t t = t0; t < nd_tasks.size(); ++t) {
-          nd_off.push_back(words[k + 1]);
-          words[k + 1] += nd_tasks[t].words;
-        }
-        flow = flow && words[k + 1] / 4 < (1ll << 31) && nd_w + nds[k].w_total < (1ll << 31);
-        nd_w += (nds[k].w_total + 63) & ~63ll;
         B.nd = 1;
         B.M = I.n1 - 1;
         B.N = I.N2;
         B.Np = (B.N + 3) & ~3;
         B.nd_depth = nds[k].depth;
-        B.foff = bcr_rows;
-        bcr_rows += (long long)B.M * B.N;
+        B.foff = fp.rows;
         B.node_off = I.node_off;
         B.nodes = I.nodes;
         B.st_off = I.lv[0].st;
-        nd_flow_places(ndu, f0, nf, (int64_t)B.M * B.N, nd_place, nd_perm);
+        flow = nd_flow_add(fp, &nds[k], (int64_t)B.M * B.N, kElem, nd_workers(kElem) * ctas, nd_vec_cap(kElem),
+                           kElem == 1 ? kNdSum8Fronts * ctas : 1 << 30);
       }
-      flow = flow && bcr_rows + nd_w < (1ll << 31) && total_nodes < (1ll << 31);
+      flow = flow && total_nodes < (1ll << 31);
       if (flow) {
         pl.bcr.nd_elem = kElem;
         size_t fr = 0, tot = 0;
         if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) fr = 0;
         cudaGetLastError();
-        const double bytes = 4.0 * (double)words[ni];
+        const double bytes = 4.0 * (double)fp.words[ni];
         pl.bcr.bytes = (int64_t)bytes;
         flow = bytes <= kBcrMaxBytes && bytes <= 0.6 * (double)fr && (bcr_nb = nd_configure(pl, sms)) > 0;
       }
       if (flow) {
-        // forward from the deepest tree level, backward from the root: every
-        // record after those it reads from
-        std::vector<int> fe, be;
-        for (size_t t = 0; t < nd_tasks.size(); ++t) (nd_tasks[t].fwd ? fe : be).push_back((int)t);
-        auto key = [&](int t) {
-          const NdFlowTask& T = nd_tasks[t];
-          return std::make_pair(T.fwd ? nds[T.inst].depth - T.level : T.level, T.inst);
-        };
-        for (std::vector<int>* v : {&fe, &be}) {
-          std::stable_sort(v->begin(), v->end(), [&](int a, int b) { return key(a) < key(b); });
-          for (int t : *v)
-            nd_list.push_back(make_int4((int)(nd_off[t] / 4), 4 * nd_tasks[t].words, nd_tasks[t].inst, nd_tasks[t].kind));
-        }
-        pl.bcr.nd_nf = (int)fe.size();
-        pl.bcr.nd_nb = (int)be.size();
-        pl.bcr.nd_stream = 4.0 * (double)words[ni] > 96.0 * 1024 * 1024;  // (L2: 129 MB)
+        bcr_rows = fp.rows;
+        nd_w = fp.w;
+        nd_flow_lists(fp);
+        pl.bcr.nd_nf = fp.nf;
+        pl.bcr.nd_nb = fp.nb;
+        pl.bcr.nd_stream = 4.0 * (double)fp.words[ni] > 96.0 * 1024 * 1024;  // (L2: 129 MB)
       } else {  // a front beyond a record or a worker's vectors: level by level (FP32), multigrid (FP64)
         pl.bcr.nd_elem = 0;
-        ndu = NdUpload();
-        nd_tasks.clear();
-        nd_off.clear();
-        nd_place.clear();
-        nd_perm.clear();
-        nd_w = 0;
-        bcr_rows = 0;
+        fp = NdFlowPlan();
       }
     }
     if (sizeof(Real) == 8) want = want && flow;
@@ -1331,36 +1324,17 @@ static int setup(apic_sim* S) {
                                               2 * kBcrMaxRhs * (size_t)(pl.bcr.chunks + ni)));
     if (pl.bcr.nd_elem > 0) {
       d.nd_rec = (const unsigned char*)d.bcr;
-      d.nd_list = (const int4*)A(sizeof(int4) * nd_list.size());
+      d.nd_list = (const int4*)A(sizeof(int4) * fp.list.size());
       d.nd_perm = (const int32_t*)A(sizeof(int32_t) * (size_t)bcr_rows);
       d.nd_w = (float*)A(E * kBcrMaxRhs * (size_t)std::max<long long>(1, nd_w));
       d.nd_e2 = A(E * kBcrMaxRhs * (size_t)bcr_rows);
       if (S->status != APIC_OK) return S->status;
-      S->h2d((int4*)d.nd_list, nd_list.data(), nd_list.size());
-      S->h2d((int32_t*)d.nd_perm, nd_perm.data(), nd_perm.size());
-      // the records, instance by instance (the host copy of one at a time)
-      std::vector<int32_t> rec;
-      for (int k = 0, t0 = 0; k < ni; ++k) {
-        int t1 = t0;
-        while (t1 < (int)nd_tasks.size() && nd_tasks[t1].inst == k) ++t1;
-        const int64_t w0 = nd_off[t0], w1 = t1 < (int)nd_tasks.size() ? nd_off[t1] : pl.bcr.bytes / 4;
+      S->h2d((NdFlowEntry*)d.nd_list, fp.list.data(), fp.list.size());
+      S->h2d((int32_t*)d.nd_perm, fp.perm.data(), fp.perm.size());
+      for (int k = 0; k < ni; ++k) {
         const NdFlowInst I{bcr_in[k].N, (int)bcr_in[k].foff, (int)bcr_in[k].node_off};
-        const NdFactor& F = nds[k];
-        rec.resize((size_t)(w1 - w0));
-        parallel_for(std::min(64, t1 - t0), [&](int q) {
-          for (int t = t0 + q; t < t1; t += std::min(64, t1 - t0)) {
-            int32_t* out = rec.data() + (nd_off[t] - w0);
-            if constexpr (sizeof(Real) == 8)
-              nd_flow_write<double>(ndu, nd_tasks[t], nd_place, nd_perm.data() + I.foff, I, F.fm64.data(), 0, F.nb64.data(), F.fm_total, out);
-            else
-              nd_flow_write<float>(ndu, nd_tasks[t], nd_place, nd_perm.data() + I.foff, I, F.fm.data(), 0,
-                                   F.nb.data(), F.fm_total, out);
-          }
-        });
-        S->h2d((int32_t*)d.bcr + w0, rec.data(), rec.size());
-        if (!S->sync()) return S->status;  // the host copies are reused or released below
+        if (!upload_records<Real>(S, fp, k, I, nds[k], (int32_t*)d.bcr)) return S->status;
         nds[k] = NdFactor();
-        t0 = t1;
       }
     } else if (!ndu.fronts.empty()) {
       d.nd_front = (const NdFront*)A(sizeof(NdFront) * ndu.fronts.size());
@@ -1836,8 +1810,6 @@ static int read_status(apic_sim* S) {
 template <class Real>
 static bool redeposit(apic_sim* S) {
   if (!S->dirty) return true;
-  if (!S->ck(cudaMemsetAsync(S->d.acc, 0, sizeof(unsigned long long) * 2 * S->d.total_nodes, S->stream), "memset"))
-    return false;
   launch_deposit_all<Real>(S->view(S->par), S->push_grid, S->max_n2, S->stream);
   S->dirty = false;
   return true;
@@ -2601,6 +2573,10 @@ static bool tangent_setup(apic_sim* S) {
   const int ni = S->n_inst;
   const size_t R = sizeof(Real);
   t.stride = S->slots;
+  // accumulators of the windows' deposits: as many as particles per node
+  S->dep_copies = (int)std::max<long long>(1, std::min<long long>(8, S->slots / tn));
+  if (S->dep_copies > 1)
+    S->dep_part = (unsigned long long*)S->dalloc(sizeof(unsigned long long) * 2 * tn * S->dep_copies);
   t.ds = S->dalloc(R * 5 * kNPar * (size_t)S->slots);
   t.drho = (double*)S->dalloc(sizeof(double) * kNPar * tn);
   t.dphi = (double*)S->dalloc(sizeof(double) * kNPar * tn);
@@ -2680,8 +2656,7 @@ static int sensitivity_impl(apic_sim* S, int n, double* values, double* jac) {
   S->ck(cudaMemsetAsync(t.vals, 0, sizeof(double) * ni * kNOut, s), "memset");
   for (int k = 0; k < n && S->status == APIC_OK; ++k) {
     // deposit of every particle (values and derivatives), charge density
-    S->ck(cudaMemsetAsync(d.acc, 0, sizeof(unsigned long long) * 2 * tn, s), "memset");
-    launch_deposit_all<Real>(d, S->push_grid, S->max_n2, s);
+    launch_deposit_all<Real>(d, S->push_grid, S->max_n2, s, S->dep_part, S->dep_copies);
     S->ck(cudaMemsetAsync(t.drho, 0, sizeof(double) * kNPar * tn, s), "memset");
     launch_tan_deposit<Real>(d, t, S->push_grid, S->max_n2, s);
     launch_rho<Real>(d, s);
@@ -2772,7 +2747,11 @@ static bool adjoint_setup(apic_sim* S, int K) {
     a.inj = (int64_t*)S->dalloc(sizeof(int64_t) * (size_t)K * S->n_pop * (size_t)a.inj_cap);
     if (!a.lam) {
       a.lam = (double*)S->dalloc(sizeof(double) * 5 * (size_t)S->slots);
-      a.lG = (double*)S->dalloc(sizeof(double) * 2 * tn);
+      // as many copies as particles per node, at most eight: the corner sums of
+      // a plasma that fills its volume meet on the outermost rows' nodes
+      a.copies = (int)std::max<long long>(1, std::min<long long>(8, S->slots / tn));
+      a.lG = (double*)S->dalloc(sizeof(double) * 2 * tn * a.copies);
+      a.sgeo = (double*)S->dalloc(sizeof(double) * 6 * (size_t)ni * (S->max_n2 + 1));
       a.lphi = (double*)S->dalloc(sizeof(double) * tn);
       a.lrho = (double*)S->dalloc(sizeof(double) * tn);
       a.Gk = S->dalloc(2 * R * tn);
@@ -2781,36 +2760,102 @@ static bool adjoint_setup(apic_sim* S, int K) {
       a.vals = (double*)S->dalloc(sizeof(double) * ni * kNOut);
     }
     if (S->status != APIC_OK) return false;
+    launch_adj_surface_geom(S->view(S->par), a, S->max_n2, S->stream);
     S->adj_K = K;
   }
-  if (a.nd_front) return true;
+  if (a.rhs) return true;
   // the transposed solve: every instance's operator (rows scaled as solved)
   // factored by nested dissection, FP64 fronts
-  NdUpload up;
   std::vector<NdFactor> fs(ni);
-  std::vector<int64_t> mat0(ni);
-  int64_t mat = 0, w = 0, unk = 0;
+  NdFlowPlan fp;
+  bool flow = true;
   int T = (int)std::min<unsigned>(16u, std::max(1u, std::thread::hardware_concurrency()));
+  if (ni > kCoopMaxInst) {
+    S->fail(APIC_ERR_INVALID_ARG, "too many instances for the reverse sweep");
+    return false;
+  }
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  double nodes = 0.0;
+  for (const Inst& I : S->inst)
+    if (!(I.flags & APIC_NO_FIELD)) nodes += (double)I.nodes;
+  std::vector<BcrInst> bi(ni, BcrInst{});
+  a.unk_off[0] = 0;
+  for (int k = 0; k < ni; ++k) {
+    const Inst& I = S->inst[k];
+    const long long unk = (long long)(I.n1 - 1) * I.N2;
+    const bool field = !(I.flags & APIC_NO_FIELD);
+    a.unk_off[k + 1] = a.unk_off[k] + unk;
+    bi[k].nd = field;
+    bi[k].M = I.n1 - 1;
+    bi[k].N = I.N2;
+    bi[k].foff = a.unk_off[k];
+    if (field) {
+      std::vector<double> V, rsc, bbc;
+      build_volumes(I, V);
+      HostLevel L;
+      build_fine(I, V, L, rsc, bbc);
+      std::string why;
+      if (!nd_build(I.n1 - 1, I.N2, nd_coef, &L, 16, T, true, fs[k], why)) {
+        S->fail(APIC_ERR_INVALID_ARG, "reverse sweep: " + why);
+        return false;
+      }
+    }
+    const int ctas = field ? std::max(1, (int)std::lround(sms * (double)I.nodes / nodes)) : 1;
+    flow = flow && nd_flow_add(fp, field ? &fs[k] : nullptr, unk, 2, nd_workers(2) * ctas, nd_vec_cap(2), 1 << 30);
+  }
+  const long long unk = a.unk_off[ni];
+  a.rhs = (double*)S->dalloc(sizeof(double) * (size_t)std::max<int64_t>(1, unk));
+  BcrPlan& b = S->adj_plan;
+  b = BcrPlan{};
+  b.nd_elem = 2;
+  int blocks = 0;
+  if (const char* e = std::getenv("APIC_ND_FLOW")) flow = flow && std::atoi(e) != 0;
+  flow = flow && (blocks = nd_transposed_configure(b, sms)) > 0;
+  if (flow) {
+    // as the solve's sweeps (nd_solve.cu), on the transposed fronts
+    nd_flow_lists(fp);
+    b.rows = fp.rows;
+    b.nd_wrows = fp.w;
+    b.nd_nf = fp.nf;
+    b.nd_nb = fp.nb;
+    b.bytes = 4 * fp.words[ni];
+    b.nd_stream = 4.0 * (double)fp.words[ni] > 96.0 * 1024 * 1024;  // (L2: 129 MB)
+    DevPtrs& v = S->adj_view;
+    int32_t* rec = (int32_t*)S->dalloc(std::max<size_t>(4, 4 * (size_t)fp.words[ni]));
+    v.nd_rec = (const unsigned char*)rec;
+    v.nd_list = (const int4*)S->dalloc(sizeof(int4) * std::max<size_t>(1, fp.list.size()));
+    v.nd_perm = (const int32_t*)S->dalloc(sizeof(int32_t) * std::max<size_t>(1, fp.perm.size()));
+    v.bcr_inst = (const BcrInst*)S->dalloc(sizeof(BcrInst) * (size_t)ni);
+    v.bcr_f = (float*)S->dalloc(sizeof(double) * (size_t)std::max<int64_t>(1, fp.rows));
+    v.bcr_e = (float*)S->dalloc(sizeof(double) * (size_t)std::max<int64_t>(1, fp.rows));
+    v.nd_e2 = S->dalloc(sizeof(double) * (size_t)std::max<int64_t>(1, fp.rows));
+    v.nd_w = (float*)S->dalloc(sizeof(double) * (size_t)std::max<int64_t>(1, fp.w));
+    v.bar = (unsigned*)S->dalloc(256);
+    if (S->status != APIC_OK) return false;
+    S->h2d((NdFlowEntry*)v.nd_list, fp.list.data(), fp.list.size());
+    S->h2d((int32_t*)v.nd_perm, fp.perm.data(), fp.perm.size());
+    S->h2d((BcrInst*)v.bcr_inst, bi.data(), bi.size());
+    for (int k = 0; k < ni; ++k) {
+      if (!bi[k].nd) continue;
+      nd_transpose64(fs[k]);
+      // the sweeps' solution is kept by unknown: rhs + foff
+      const NdFlowInst I{bi[k].N, (int)bi[k].foff, (int)bi[k].foff - bi[k].N};
+      if (!upload_records<double>(S, fp, k, I, fs[k], rec)) return false;
+      fs[k] = NdFactor();
+    }
+    S->adj_blocks = blocks;
+    return S->sync();
+  }
+  // a front beyond a record: one launch per tree level
+  NdUpload up;
+  std::vector<int64_t> mat0(ni);
+  int64_t mat = 0, w = 0;
   S->adj_levels.assign(ni, {});
   S->adj_smem.assign(ni, 1);
   for (int k = 0; k < ni; ++k) {
-    const Inst& I = S->inst[k];
-    if (ni > kCoopMaxInst) {
-      S->fail(APIC_ERR_INVALID_ARG, "too many instances for the reverse sweep");
-      return false;
-    }
-    a.unk_off[k] = unk;
-    unk += (long long)(I.n1 - 1) * I.N2;
-    if (I.flags & APIC_NO_FIELD) continue;
-    std::vector<double> V, rsc, bbc;
-    build_volumes(I, V);
-    HostLevel L;
-    build_fine(I, V, L, rsc, bbc);
-    std::string why;
-    if (!nd_build(I.n1 - 1, I.N2, nd_coef, &L, 16, T, true, fs[k], why)) {
-      S->fail(APIC_ERR_INVALID_ARG, "reverse sweep: " + why);
-      return false;
-    }
+    if (!bi[k].nd) continue;
     const int f0 = (int)up.fronts.size();
     NdLevels lv;
     nd_layout(fs[k], mat, w, kNdWarpMaxS, kNdWarpMaxU, kNdWarpStage, kNdTaskFloats, kNdTaskRows, kNdTaskFronts,
@@ -2828,8 +2873,6 @@ static bool adjoint_setup(apic_sim* S, int K) {
       S->adj_smem[k] = std::max(S->adj_smem[k], F.s + F.u);
     }
   }
-  a.unk_off[ni] = unk;
-  a.rhs = (double*)S->dalloc(sizeof(double) * (size_t)std::max<int64_t>(1, unk));
   a.ndw = (double*)S->dalloc(sizeof(double) * (size_t)std::max<int64_t>(1, w));
   double* mbuf = (double*)S->dalloc(sizeof(double) * (size_t)std::max<int64_t>(1, mat));
   a.nd_front = (const NdFront*)S->dalloc(sizeof(NdFront) * std::max<size_t>(1, up.fronts.size()));
@@ -2870,34 +2913,32 @@ static int adjoint_impl(apic_sim* S, int n, const double* dL_dout, double* value
   const int ni = S->n_inst;
   cudaStream_t s = S->stream;
   const size_t R = sizeof(Real);
-  const size_t pbytes = R * (size_t)S->slots;
   std::vector<double> seed((size_t)ni * kNOut);
   for (size_t q = 0; q < seed.size(); ++q) seed[q] = dL_dout[q] / n;
   S->h2d(a.seed, seed.data(), seed.size());
   S->ck(cudaMemsetAsync(a.grad, 0, sizeof(double) * ni * kNPar, s), "memset");
   S->ck(cudaMemsetAsync(a.vals, 0, sizeof(double) * ni * kNOut, s), "memset");
   S->ck(cudaMemsetAsync(a.inj, 0xff, sizeof(int64_t) * (size_t)n * S->n_pop * a.inj_cap, s), "memset");
-  void* arr[5] = {d.x1, d.x2, d.vR, d.vZ, d.vT};
-  // forward pass, checkpoint k holding the state at the start of step k
+  // forward pass, checkpoint k holding the state at the start of step k (the
+  // particles' written by the push as it reads them)
   for (int k = 0; k < n && S->status == APIC_OK; ++k) {
-    for (int c = 0; c < 5; ++c)
-      S->ck(cudaMemcpyAsync((char*)a.ck + ((size_t)k * 5 + c) * pbytes, arr[c], pbytes, cudaMemcpyDeviceToDevice, s),
-            "checkpoint");
     S->ck(cudaMemcpyAsync(a.ck_ps + (size_t)k * S->n_pop, d.ps, sizeof(PopState) * S->n_pop, cudaMemcpyDeviceToDevice,
                           s),
           "checkpoint");
-    S->ck(cudaMemsetAsync(d.acc, 0, sizeof(unsigned long long) * 2 * tn, s), "memset");
-    launch_deposit_all<Real>(d, S->push_grid, S->max_n2, s);
-    launch_rho<Real>(d, s);
+    launch_deposit_all<Real>(d, S->push_grid, S->max_n2, s, S->dep_part, S->dep_copies);
+    if (S->plan.bcr.n_inst > 0) {  // density, solve and fields in one launch
+      if (!S->ck(solve_coop<Real>(S, d, s, kBcrRho | kBcrFields), "cooperative solve")) break;
+    } else {
+      launch_rho<Real>(d, s);
+      if (!solve_now<Real>(S, d)) break;
+      launch_gradients<Real>(d, s);
+      launch_surface(d, s);
+    }
     S->ck(cudaMemcpyAsync(a.ck_rho + (size_t)k * tn, d.rho, sizeof(double) * tn, cudaMemcpyDeviceToDevice, s), "ck");
-    if (!solve_now<Real>(S, d)) break;
     S->ck(cudaMemcpyAsync(a.ck_phi + (size_t)k * tn, d.phi, sizeof(double) * tn, cudaMemcpyDeviceToDevice, s), "ck");
-    launch_gradients<Real>(d, s);
-    launch_surface(d, s);
     launch_adj_fwd_push<Real>(d, a, k, s);
     launch_adj_fwd_inject<Real>(d, a, t, k, S->max_inj, s);
-    launch_adj_values(d, a, s);
-    launch_step_end(d, s);
+    launch_step_end(d, s, a.vals);
     S->host_step += 1;
   }
   S->ck(cudaMemcpyAsync(a.ck_ps + (size_t)n * S->n_pop, d.ps, sizeof(PopState) * S->n_pop, cudaMemcpyDeviceToDevice, s),
@@ -2910,19 +2951,34 @@ static int adjoint_impl(apic_sim* S, int n, const double* dL_dout, double* value
     dg.phi = a.ck_phi + (size_t)k * tn;
     dg.G = a.Gk;
     launch_gradients<Real>(dg, s);
-    S->ck(cudaMemsetAsync(a.lG, 0, sizeof(double) * 2 * tn, s), "memset");
+    S->ck(cudaMemsetAsync(a.lG, 0, sizeof(double) * 2 * tn * a.copies, s), "memset");
     S->ck(cudaMemsetAsync(a.lphi, 0, sizeof(double) * tn, s), "memset");
     launch_adj_rev_inject<Real>(d, a, t, k, S->max_inj, s);
     launch_adj_rev_push<Real>(d, a, t, k, s);
-    launch_adj_surface(d, a, t, k, s);
+    launch_adj_surface(d, a, k, S->max_n2, s);
     launch_adj_gradT(d, a, s);
-    launch_adj_to_unknowns(d, a, s);
-    for (int q = 0; q < ni; ++q) {
-      const auto& lv = S->adj_levels[q];
-      for (int l = (int)lv.size() - 1; l >= 0; --l)
-        launch_adj_ndT(a, lv[l].first, lv[l].second, a.unk_off[q], S->adj_smem[q], true, s);
-      for (int l = 0; l < (int)lv.size(); ++l)
-        launch_adj_ndT(a, lv[l].first, lv[l].second, a.unk_off[q], S->adj_smem[q], false, s);
+    if (S->adj_blocks > 0) {
+      DevPtrs v = d;
+      const DevPtrs& w = S->adj_view;
+      v.nd_rec = w.nd_rec;
+      v.nd_list = w.nd_list;
+      v.nd_perm = w.nd_perm;
+      v.bcr_inst = w.bcr_inst;
+      v.bcr_f = w.bcr_f;
+      v.bcr_e = w.bcr_e;
+      v.nd_e2 = w.nd_e2;
+      v.nd_w = w.nd_w;
+      v.bar = w.bar;  // (its own barrier counter: another number of CTAs than the solve's)
+      if (!S->ck(launch_nd_transposed(v, S->adj_plan, S->adj_blocks, a.lphi, a.rhs, s), "transposed solve")) break;
+    } else {
+      launch_adj_to_unknowns(d, a, s);
+      for (int q = 0; q < ni; ++q) {
+        const auto& lv = S->adj_levels[q];
+        for (int l = (int)lv.size() - 1; l >= 0; --l)
+          launch_adj_ndT(a, lv[l].first, lv[l].second, a.unk_off[q], S->adj_smem[q], true, s);
+        for (int l = 0; l < (int)lv.size(); ++l)
+          launch_adj_ndT(a, lv[l].first, lv[l].second, a.unk_off[q], S->adj_smem[q], false, s);
+      }
     }
     launch_adj_after_solve(d, a, t, k, s);
     launch_adj_rev_deposit<Real>(d, a, k, s);

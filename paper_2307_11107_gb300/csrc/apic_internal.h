@@ -258,7 +258,7 @@ struct TanPtrs {
 // pass then runs the step's operations backwards, from step K-1 to 0.
 struct AdjPtrs {
   int K;                   // window steps
-  int pad;
+  int copies;
   int64_t stride;          // particle slots of one component (all populations)
   void* ck;                // [K][5][stride] particle state at the start of step k (particle precision)
   PopState* ck_ps;         // [K + 1][n_pop] population counters at the start of step k (k = K: after the window)
@@ -269,12 +269,13 @@ struct AdjPtrs {
                            // -1 absorbed during its first flight, -2 escaped
   int64_t inj_cap;
   double* lam;             // [5][stride] adjoint of the particle state
-  double* lG;              // [2][total_nodes] adjoint of the node gradients
+  double* lG;              // [copies][2][total_nodes] adjoint of the node gradients (a CTA adds to one copy)
   double* lphi;            // [total_nodes] adjoint of phi
   double* lrho;            // [total_nodes] adjoint of rho
   double* rhs;             // transposed solve: right-hand side / solution over every instance's unknowns
   double* ndw;             // its update vectors
   void* Gk;                // node gradients of step k (pairs of the particle type)
+  double* sgeo;            // [n_inst][n2_max + 1][6] grain surface constants
   double* seed;            // [n_inst][kNOut] dL / d(output of one step) = dL_dout / K
   double* grad;            // [n_inst][kNPar] parameter adjoints
   double* vals;            // [n_inst][kNOut] window sums of the outputs
@@ -285,7 +286,7 @@ struct AdjPtrs {
   const double* nd_mat;
   int64_t unk_off[kCoopMaxInst + 1];  // first unknown of each instance in rhs
 };
-constexpr int kAdjBlocks = 256;  // CTAs of the reverse particle kernels (fixed: deterministic partial sums)
+constexpr int kAdjBlocks = 1216;  // CTAs of the reverse particle kernels at most (eight per SM)
 
 // ---- launchers (defined in the kernel translation units) ----
 template <class Real>
@@ -294,8 +295,11 @@ void launch_load(const DevPtrs& d, int pop, long long n0, long long count, long 
 template <class Real>
 void launch_explicit(const DevPtrs& d, int pop, long long n0, long long count, const double* dstate,
                      cudaStream_t s);
+// clears the accumulator first; part: `copies` accumulators of the caller's to
+// share out the additions, or null
 template <class Real>
-void launch_deposit_all(const DevPtrs& d, int max_grid, int max_n2, cudaStream_t s);
+void launch_deposit_all(const DevPtrs& d, int max_grid, int max_n2, cudaStream_t s, unsigned long long* part = nullptr,
+                        int copies = 1);
 #ifndef APIC_PUSH4_MIN_BLOCKS
 #define APIC_PUSH4_MIN_BLOCKS 3  // CTAs of the vector push per SM (80 registers: the four particles stay in registers)
 #endif
@@ -329,7 +333,8 @@ void launch_rho(const DevPtrs& d, cudaStream_t s);
 template <class Real>
 void launch_gradients(const DevPtrs& d, cudaStream_t s);
 void launch_surface(const DevPtrs& d, cudaStream_t s);
-void launch_step_end(const DevPtrs& d, cudaStream_t s);
+// vals: window sums of the step's outputs to add to (adjoint window), or null
+void launch_step_end(const DevPtrs& d, cudaStream_t s, double* vals = nullptr);
 void launch_b_from_rho(const DevPtrs& d, int inst, cudaStream_t s);
 void launch_b_vacuum(const DevPtrs& d, int inst, cudaStream_t s);
 void launch_store_vacuum(const DevPtrs& d, int inst, cudaStream_t s);
@@ -393,6 +398,7 @@ constexpr int kNdStageFloats = 16 * kNdWarpStage;  // the CTA's stage
 constexpr int kNdUnitStage = kNdStageFloats / kNdUnits;  // a task's staged matrix rows at most
 constexpr int kNdTaskFloats = kNdUnitStage;  // matrix floats per task of a large front (row chunks)
 constexpr int kNdTaskFronts = 16 / kNdUnits;  // small fronts per task at most (one per warp of a worker)
+constexpr int kNdSum8Fronts = 16;    // nd_flow_tasks's sum8, per CTA of an instance's share
 constexpr int kNdTaskRows = 2048 / kNdUnits;  // rows per task of a large front at most
 static_assert((kNdUnits == 1 || kNdUnits == 2 || kNdUnits == 4 || kNdUnits == 8) &&
                   kNdWarpStage * kNdTaskFronts <= kNdUnitStage,
@@ -510,6 +516,11 @@ const void* bcr_kernel(const SolvePlan& plan);  // the solve kernel (to find its
 // co-residable; sets plan.bcr.dyn) and the longest vector of a front it takes
 const void* nd_kernel(const SolvePlan& plan);
 int nd_configure(SolvePlan& plan, int sms);
+// The reverse sweep's transposed solve (FP64 records of the transposed
+// fronts): CTAs (0: not co-residable) and dynamic shared memory in b.dyn.
+int nd_transposed_configure(BcrPlan& b, int sms);
+cudaError_t launch_nd_transposed(const DevPtrs& d, const BcrPlan& b, int blocks, const double* lphi, double* out,
+                                 cudaStream_t s);
 int nd_vec_cap(int elem);
 // Workers of 128 threads per CTA of the dataflow solve.
 constexpr int nd_workers(int elem) { return elem == 2 ? 4 : 6; }
@@ -550,8 +561,8 @@ template <class Real>
 void launch_adj_rev_push(const DevPtrs& d, const AdjPtrs& a, const TanPtrs& t, int k, cudaStream_t s);
 template <class Real>
 void launch_adj_rev_deposit(const DevPtrs& d, const AdjPtrs& a, int k, cudaStream_t s);
-void launch_adj_values(const DevPtrs& d, const AdjPtrs& a, cudaStream_t s);
-void launch_adj_surface(const DevPtrs& d, const AdjPtrs& a, const TanPtrs& t, int k, cudaStream_t s);
+void launch_adj_surface_geom(const DevPtrs& d, const AdjPtrs& a, int n2_max, cudaStream_t s);
+void launch_adj_surface(const DevPtrs& d, const AdjPtrs& a, int k, int n2_max, cudaStream_t s);
 void launch_adj_gradT(const DevPtrs& d, const AdjPtrs& a, cudaStream_t s);
 void launch_adj_to_unknowns(const DevPtrs& d, const AdjPtrs& a, cudaStream_t s);
 // the transposed sweeps over one tree level's fronts [f0, f1) of the instance

@@ -193,7 +193,7 @@ __device__ void finish_injection(PopState& S, const Pop& P) {
   S.inj_stored = 0;
 }
 
-__global__ void k_step_end(DevPtrs d) {
+__global__ void k_step_end(DevPtrs d, double* vals) {
   const int inst = blockIdx.x * blockDim.x + threadIdx.x;
   if (inst >= d.n_inst) return;
   const Inst& I = d.inst[inst];
@@ -227,6 +227,14 @@ __global__ void k_step_end(DevPtrs d) {
   h[8] = res[1];
   h[9] = T.tally[4];
   h[10] = (I.flags & APIC_FLOATING) ? T.phig : I.phi_g;
+  if (vals) {
+    double* v = vals + (long long)inst * kNOut;
+    v[0] += T.tally[1] / dt;
+    v[1] += T.FZ;
+    v[2] += T.tally[0] / dt;
+    v[3] += T.tally[2] / dt;
+    v[4] += T.Q;
+  }
   if (I.flags & APIC_FLOATING) T.qg += T.tally[0];  // charge the grain collected this step
   for (int k = 0; k < 5; ++k) T.tally[k] = 0.0;
   T.step += 1;
@@ -253,7 +261,9 @@ template void launch_gradients<double>(const DevPtrs&, cudaStream_t);
 template void launch_gradients<float>(const DevPtrs&, cudaStream_t);
 
 void launch_surface(const DevPtrs& d, cudaStream_t s) { k_surface<<<d.n_inst, 256, 0, s>>>(d); }
-void launch_step_end(const DevPtrs& d, cudaStream_t s) { k_step_end<<<(d.n_inst + 63) / 64, 64, 0, s>>>(d); }
+void launch_step_end(const DevPtrs& d, cudaStream_t s, double* vals) {
+  k_step_end<<<(d.n_inst + 63) / 64, 64, 0, s>>>(d, vals);
+}
 void launch_finish_injection(const DevPtrs& d, int pop, cudaStream_t s) { k_finish_injection<<<1, 1, 0, s>>>(d, pop); }
 void launch_b_from_rho(const DevPtrs& d, int inst, cudaStream_t s) { k_b_from_rho<<<kRedBlocks, 256, 0, s>>>(d, inst); }
 void launch_b_vacuum(const DevPtrs& d, int inst, cudaStream_t s) { k_b_vacuum<<<kRedBlocks, 256, 0, s>>>(d, inst); }

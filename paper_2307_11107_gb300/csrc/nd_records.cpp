@@ -7,6 +7,8 @@
 namespace apic {
 namespace {
 
+constexpr int kWarpS = 64, kWarpU = 192;  // a warp's vector areas
+
 bool has_gather(const NdFront& F) { return F.child[0] >= 0 || F.child[1] >= 0; }
 
 // Shape of a task's dot products: vectors of a row, lanes per row (as a power
@@ -51,9 +53,8 @@ int rows_of(const NdFront& F, bool fwd) { return fwd ? F.s + F.u : F.s; }
 
 bool nd_flow_tasks(const NdUpload& up, int front0, int nf, int depth, int inst, bool fwd, int elem, int units,
                    int vec_cap, int sum8, std::vector<NdFlowTask>& tasks) {
-  const int kMaxS = 64, kMaxU = 192;  // a warp's vector areas
   auto large = [&](const NdFront& F) {
-    return F.s > kMaxS || F.u > kMaxU ||
+    return F.s > kWarpS || F.u > kWarpU ||
            4 * rows_of(F, fwd) * shape_of(F, fwd, elem, false).stride > kNdFlowWarpWords;
   };
   auto tiny0 = [&](const NdFront& F) { return F.s <= kNdTinyS && F.u <= kNdTinyU && !large(F); };
@@ -129,6 +130,56 @@ void nd_flow_places(const NdUpload& up, int front0, int nf, int64_t unknowns, st
     place.push_back(p);
     for (int a = 0; a < F.s; ++a) perm[base + up.idx[F.S + a]] = p + a;
     p += F.s;
+  }
+}
+
+bool nd_flow_add(NdFlowPlan& P, const NdFactor* f, int64_t unknowns, int elem, int units, int vec_cap, int sum8) {
+  const int inst = (int)P.depth.size(), f0 = (int)P.up.fronts.size();
+  P.words.push_back(P.words.back());
+  P.depth.push_back(f ? f->depth : 0);
+  bool ok = true;
+  if (f) {
+    NdLevels lv;
+    nd_layout(*f, 0, P.w, kWarpS, kWarpU, 2048, 8192, 512, 4, 8192, 1, P.up, lv);  // (its level-by-level tasks are not used)
+    const size_t t0 = P.tasks.size();
+    for (int sw = 0; sw < 2 && ok; ++sw)
+      ok = nd_flow_tasks(P.up, f0, (int)P.up.fronts.size() - f0, f->depth, inst, sw == 0, elem, units, vec_cap, sum8,
+                         P.tasks);
+    for (size_t t = t0; t < P.tasks.size(); ++t) {
+      P.off.push_back(P.words.back());
+      P.words.back() += P.tasks[t].words;
+    }
+    P.w += (f->w_total + 63) & ~63ll;
+  }
+  nd_flow_places(P.up, f0, (int)P.up.fronts.size() - f0, unknowns, P.place, P.perm);
+  P.rows += unknowns;
+  return ok && P.words.back() / 4 < (1ll << 31) && P.rows + P.w < (1ll << 31);
+}
+
+void nd_flow_lists(NdFlowPlan& P) {
+  std::vector<int> v[2];
+  for (size_t t = 0; t < P.tasks.size(); ++t) v[P.tasks[t].fwd ? 0 : 1].push_back((int)t);
+  auto key = [&](int t) {
+    const NdFlowTask& T = P.tasks[t];
+    return std::make_pair(T.fwd ? P.depth[T.inst] - T.level : T.level, T.inst);
+  };
+  P.list.clear();
+  for (std::vector<int>& q : v) {
+    std::stable_sort(q.begin(), q.end(), [&](int a, int b) { return key(a) < key(b); });
+    for (int t : q)
+      P.list.push_back(NdFlowEntry{(int)(P.off[t] / 4), 4 * P.tasks[t].words, P.tasks[t].inst, P.tasks[t].kind});
+  }
+  P.nf = (int)v[0].size();
+  P.nb = (int)v[1].size();
+}
+
+void nd_transpose64(NdFactor& f) {
+  for (const NdFront& F : f.fronts) {
+    double *a = f.fm64.data() + F.FM, *b = f.nb64.data() + F.NB;
+    for (int r = 0; r < F.s; ++r)
+      for (int c = 0; c < r; ++c) std::swap(a[(int64_t)r * F.sp + c], a[(int64_t)c * F.sp + r]);
+    for (int r = 0; r < F.s; ++r)
+      for (int q = 0; q < F.u; ++q) std::swap(b[(int64_t)r * F.up + q], a[(int64_t)(F.s + q) * F.sp + r]);
   }
 }
 
@@ -220,7 +271,7 @@ int64_t nd_flow_solve_host(const std::vector<int32_t>& rec, const std::vector<in
         if (!((lg == 0 && (sum == 2 || sum == 3)) || (lg == 1 && sum == 4) || (sum == 5 && (lg == 2 || lg == 5)))) return -1;
         if (sum == 2 && E[kNdVecs] > 4) return -1;
         if (R[0] == 2 && (s > kNdTinyS || u > kNdTinyU)) return -1;
-        if (R[0] == 1 && (s > 64 || u > 192)) return -1;
+        if (R[0] == 1 && (s > kWarpS || u > kWarpU)) return -1;
         if (R[0] == 0 && nr > kNdFlowRows) return -1;
         for (int q = 0; q < 2; ++q) {
           const int rp = E[kNdRep0 + q];

@@ -79,6 +79,39 @@ void nd_flow_write(const NdUpload& up, const NdFlowTask& T, const std::vector<in
                    const NdFlowInst& I, const M* fm,
                    int64_t fm0, const M* nb, int64_t nb0, int32_t* out);
 
+// A list entry, same layout as CUDA's int4: a record's first word / 4, its
+// bytes, instance and kind.
+struct NdFlowEntry {
+  int at, bytes, inst, kind;
+};
+
+// The records of a batch: instances are added in order, then the lists made.
+struct NdFlowPlan {
+  NdUpload up;
+  std::vector<NdFlowTask> tasks;        // instance by instance
+  std::vector<int64_t> off;             // their first words
+  std::vector<int64_t> words{0};        // first word of each instance's records (and the end)
+  std::vector<int32_t> place, perm;     // nd_flow_places
+  std::vector<int> depth;               // of each instance's tree
+  std::vector<NdFlowEntry> list;        // the forward sweep's entries, then the backward one's
+  int nf = 0, nb = 0;
+  int64_t rows = 0, w = 0;              // unknowns and update-vector entries so far
+};
+
+// Adds f as the next instance (its right-hand side at P.rows, its update
+// vectors at P.w); unknowns: M N, also where the instance has no fronts (f
+// null).  False: a front does not fit, or an offset exceeds 31 bits.
+bool nd_flow_add(NdFlowPlan& P, const NdFactor* f, int64_t unknowns, int elem, int units, int vec_cap, int sum8);
+
+// The lists, forward from the deepest tree level, backward from the root:
+// every record after those it reads from.
+void nd_flow_lists(NdFlowPlan& P);
+
+// The fronts of the transposed system in place (FP64): those of A^T are the
+// transposes of A's, F_SS^-T and, as the lower block, (F_SS^-1 F_SU)^T; the
+// lower block's transpose in place of F_SS^-1 F_SU.
+void nd_transpose64(NdFactor& f);
+
 // The sweeps as the device runs them, record by record in list order (offsets
 // in words into rec): f in places, x += A^-1 f for the unknowns of every
 // instance, w: the update vectors' total.  Returns the entries that were read

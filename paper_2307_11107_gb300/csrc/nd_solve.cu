@@ -579,6 +579,41 @@ k_solve_nd(const __grid_constant__ DevPtrs d, const __grid_constant__ BcrPlan pl
   }
 }
 
+// lambda_b = A^-T lambda_phi for the reverse sweep (adjoint.cu): the records
+// hold the transposed fronts.  lphi: by node; out: by unknown (from each
+// instance's foff).  256 x 128: 88 us, with one launch per tree level (28 of
+// them, a CTA per front) 840.
+__global__ void __launch_bounds__(nd_threads(2), 1)
+k_nd_transposed(const __grid_constant__ DevPtrs d, const __grid_constant__ BcrPlan pl, const double* lphi,
+                const __grid_constant__ BcrRhs rhs) {
+  constexpr int kWk = nd_workers(2);
+  extern __shared__ __align__(128) char s_dyn[];
+  __shared__ int s_act[kCoopMaxInst];
+  __shared__ __align__(8) uint64_t s_bar[kWk];
+  const int nb = gridDim.x, ni = d.n_inst;
+  for (int k = threadIdx.x; k < ni; k += blockDim.x) s_act[k] = 1;
+  if (threadIdx.x < kWk) mbar_init(&s_bar[threadIdx.x], 1);
+  const int t = blockIdx.x * (int)blockDim.x + threadIdx.x, nt = nb * (int)blockDim.x;
+  for (int k = 0; k < ni; ++k) {
+    const BcrInst& B = d.bcr_inst[k];
+    if (!B.nd) continue;
+    const double* src = lphi + d.inst[k].node_off + B.N;
+    for (int z = t; z < B.M * B.N; z += nt) {
+      ((double*)d.bcr_f)[B.foff + d.nd_perm[B.foff + z]] = src[z];
+      rhs.x[0][B.foff + z] = 0.0;
+    }
+  }
+  for (int z = t; z < (int)pl.rows; z += nt) ((double*)d.nd_e2)[z] = Dyn<double>::mark();
+  for (int z = t; z < (int)pl.nd_wrows; z += nt) ((double*)d.nd_w)[z] = Dyn<double>::mark();
+  if (!grid_sync(d, nb)) return;
+  const int h = (int)threadIdx.x / kWkThreads;
+  char* wk = s_dyn + h * kWkBytes;
+  unsigned copies = 0;
+  sweep<double, true>(d, pl, d.nd_list, pl.nd_nf, 1, s_act, wk, s_bar + h, copies, rhs);
+  if (!grid_sync(d, nb)) return;
+  sweep<double, false>(d, pl, d.nd_list + pl.nd_nf, pl.nd_nb, 1, s_act, wk, s_bar + h, copies, rhs);
+}
+
 const void* kernel_of(const BcrPlan& b) {
   return b.nd_elem == 2 ? (const void*)k_solve_nd<double> : (const void*)k_solve_nd<float>;
 }
@@ -589,18 +624,30 @@ const void* nd_kernel(const SolvePlan& pl) { return kernel_of(pl.bcr); }
 
 int nd_vec_cap(int elem) { return elem == 2 ? vec_cap<double>() : vec_cap<float>(); }
 
-int nd_configure(SolvePlan& pl, int sms) {
-  const void* kern = kernel_of(pl.bcr);
-  const int threads = nd_threads(pl.bcr.nd_elem);
-  pl.bcr.dyn = nd_workers(pl.bcr.nd_elem) * kWkBytes;
+static int configure(const void* kern, BcrPlan& b, int sms) {
+  b.dyn = nd_workers(b.nd_elem) * kWkBytes;
   int per_sm = 0;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, pl.bcr.dyn) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, (size_t)pl.bcr.dyn) != cudaSuccess ||
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, b.dyn) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nd_threads(b.nd_elem), (size_t)b.dyn) != cudaSuccess ||
       per_sm < 1) {
     cudaGetLastError();
     return 0;
   }
   return sms < kCoopMaxBlocks ? sms : kCoopMaxBlocks;
+}
+
+int nd_configure(SolvePlan& pl, int sms) { return configure(kernel_of(pl.bcr), pl.bcr, sms); }
+
+int nd_transposed_configure(BcrPlan& b, int sms) { return configure((const void*)k_nd_transposed, b, sms); }
+
+cudaError_t launch_nd_transposed(const DevPtrs& d, const BcrPlan& b, int blocks, const double* lphi, double* out,
+                                 cudaStream_t s) {
+  BcrRhs rhs{};
+  rhs.n = 1;
+  rhs.x[0] = out;
+  void* args[] = {(void*)&d, (void*)&b, (void*)&lphi, (void*)&rhs};
+  return cudaLaunchCooperativeKernel((const void*)k_nd_transposed, dim3(blocks), dim3(nd_threads(2)), args,
+                                     (size_t)b.dyn, s);
 }
 
 }  // namespace apic

@@ -1026,8 +1026,16 @@ __global__ void __launch_bounds__(256, APIC_PUSH4_MIN_BLOCKS) k_push4(DevPtrs d,
 // of one population, flushed to the global accumulator only when a chunk's
 // first row or population leaves it; corners outside the window go to global
 // memory directly.  Integer sums: the result does not depend on the order.
+// Unsorted particles all go to global memory, and those of a plasma that
+// fills its volume mostly to the outermost rows, where the additions to a node
+// follow one another at L2; so the CTAs share out `copies` accumulators,
+// `stride` apart from `acc` on, where the caller keeps them (the windows, with
+// a deposit in every step; added up by k_fold_acc).  2e6 unsorted particles on
+// 256 x 128 cells: 94 us with one, 71 and 4 for the sum with eight.
 constexpr int kDepItems = 8;
-__global__ void __launch_bounds__(256) k_deposit_all(DevPtrs d, int win_n2) {
+__global__ void __launch_bounds__(256) k_deposit_all(DevPtrs d, int win_n2, unsigned long long* acc, long long stride,
+                                                     int copies) {
+  acc += stride * (blockIdx.x % (unsigned)copies);
   extern __shared__ unsigned long long s_dw[];  // [kWinRows][win_n2 + 1]
   __shared__ long long s_pre[kMaxPop + 1];
   __shared__ int s_row0, s_wpop, s_newrow0, s_newpop, s_flush;
@@ -1054,7 +1062,7 @@ __global__ void __launch_bounds__(256) k_deposit_all(DevPtrs d, int win_n2) {
     const Pop& P = d.pop[wp];
     const Inst& I = d.inst[P.inst];
     const int rows = I.n2 <= win_n2 ? kWinRows : 0;
-    unsigned long long* g = d.acc + P.acc_off;
+    unsigned long long* g = acc + P.acc_off;
     for (int e = threadIdx.x; e < rows * I.N2; e += blockDim.x) {
       const int r = e / I.N2, j = e - r * I.N2;
       const unsigned long long v = s_dw[r * WN + j];
@@ -1112,7 +1120,7 @@ __global__ void __launch_bounds__(256) k_deposit_all(DevPtrs d, int win_n2) {
         if (w.w01) atomicAdd(sw + 1, w.w01);
         if (w.w11) atomicAdd(sw + WN + 1, w.w11);
       } else {
-        unsigned long long* g = d.acc + dep_key(I, P, c);
+        unsigned long long* g = acc + dep_key(I, P, c);
         if (w.w00) atomicAdd(g, w.w00);
         if (w.w10) atomicAdd(g + I.N2, w.w10);
         if (w.w01) atomicAdd(g + 1, w.w01);
@@ -1122,6 +1130,16 @@ __global__ void __launch_bounds__(256) k_deposit_all(DevPtrs d, int win_n2) {
     __syncthreads();
   }
   if (s_wpop >= 0) flush(s_wpop, s_row0);
+}
+
+__global__ void __launch_bounds__(256) k_fold_acc(unsigned long long* acc, const unsigned long long* part, long long n,
+                                                  int copies) {
+  for (long long z = (long long)blockIdx.x * blockDim.x + threadIdx.x; z < n; z += (long long)gridDim.x * blockDim.x) {
+    unsigned long long v = 0;
+#pragma unroll 4
+    for (int c = 0; c < copies; ++c) v += part[c * n + z];
+    acc[z] = v;
+  }
 }
 
 // Initial load, uniform in physical volume: x2 from the inverse CDF of
@@ -1750,11 +1768,15 @@ void launch_explicit<Real>(const DevPtrs& d, int pop, long long n0, long long co
 }
 
 template <>
-void launch_deposit_all<Real>(const DevPtrs& d, int max_grid, int max_n2, cudaStream_t s) {
+void launch_deposit_all<Real>(const DevPtrs& d, int max_grid, int max_n2, cudaStream_t s, unsigned long long* part,
+                              int copies) {
+  const long long n = 2 * d.total_nodes;
+  cudaMemsetAsync(part ? part : d.acc, 0, sizeof(unsigned long long) * n * (part ? copies : 1), s);
   const int win_n2 = max_n2 < kWinMaxN2 - 1 ? max_n2 : kWinMaxN2 - 1;
   const int sm = kWinRows * (win_n2 + 1) * (int)sizeof(unsigned long long);
   cudaFuncSetAttribute(k_deposit_all, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  k_deposit_all<<<max_grid, 256, sm, s>>>(d, win_n2);
+  k_deposit_all<<<max_grid, 256, sm, s>>>(d, win_n2, part ? part : d.acc, n, part ? copies : 1);
+  if (part) k_fold_acc<<<blocks_for(n, 256), 256, 0, s>>>(d.acc, part, n, copies);
 }
 
 // Dynamic shared memory of the push: window, chunk prefix, population constants.
