@@ -208,21 +208,27 @@ struct DevPtrs {
 };
 
 #ifdef __CUDACC__
-// This step's tallies of instance `inst` from its populations' fixed-point
-// sums, in population order: charge, p_Z, L_z, heat (E_kin + E_bind), events.
-__device__ inline void step_tallies(const DevPtrs& d, int inst, double out[5]) {
-  const Inst& I = d.inst[inst];
-  for (int k = 0; k < 5; ++k) out[k] = 0.0;
+// This step's tally k of instance I from its populations' fixed-point sums, in
+// population order: charge, p_Z, L_z, heat (E_kin + E_bind), events.
+__device__ inline double step_tally(const DevPtrs& d, const Inst& I, int k) {
+  double out = 0.0;
   for (int s = 0; s < I.n_species; ++s) {
     const Pop& P = d.pop[I.pop0 + s];
     const unsigned long long* st = d.tfix + P.tfix_off + (long long)I.n2 * kTallyBinWords;
     const double hits = (double)st[0], mwu = P.m * P.w * P.tunit;
-    out[0] += hits * P.q * P.w;
-    out[1] += mwu * fixed128_value(st[1], st[2]);
-    out[2] += mwu * fixed128_value(st[3], st[4]);
-    out[3] += mwu * P.tunit * fixed128_value(st[5], st[6]) + (P.q > 0.0 ? hits * I.e_bind * P.w : 0.0);
-    out[4] += hits;
+    if (k == 0) {
+      out += hits * P.q * P.w;
+    } else if (k == 4) {
+      out += hits;
+    } else {
+      const double v = fixed128_value(st[2 * k - 1], st[2 * k]);
+      out += k < 3 ? mwu * v : mwu * P.tunit * v + (P.q > 0.0 ? hits * I.e_bind * P.w : 0.0);
+    }
   }
+  return out;
+}
+__device__ inline void step_tallies(const DevPtrs& d, int inst, double out[5]) {
+  for (int k = 0; k < 5; ++k) out[k] = step_tally(d, d.inst[inst], k);
 }
 #endif
 
