@@ -2178,7 +2178,10 @@ extern "C" int apic_tallies(apic_sim* S, int32_t instance, apic_tallies_t* out) 
   S->d2h((StepState*)(S->h_tally + o_stp), S->d.stp + instance, 1);
   S->d2h((SolverState*)(S->h_tally + o_sol), S->d.sol + instance, 1);
   S->d2h(psd, S->d.ps + I.pop0, (size_t)I.n_species);  // the instance's populations are consecutive
-  S->d2h(hist, S->d.hist + I.hist_off, nh);
+  // the history's rows so far (a young run's are a small part of the ring:
+  // 4096 rows are 360 KB, 10 us of a 32 x 16 step's 140)
+  const long long have = out->history ? std::min<long long>(S->host_step, I.hist_cap) : 0;
+  if (have > 0) S->d2h(hist, S->d.hist + I.hist_off, (size_t)have * kNH);
   if (!S->sync()) return S->status;
   StepState stp;
   SolverState sol;
@@ -2222,6 +2225,7 @@ extern "C" int apic_tallies(apic_sim* S, int32_t instance, apic_tallies_t* out) 
   out->poisson_res = sol.res;
   out->poisson_iters = sol.iters;
   long long rows = std::min<long long>(stp.step, I.hist_cap);
+  if (out->history && rows > have && (!S->d2h(hist, S->d.hist + I.hist_off, nh) || !S->sync())) return S->status;
   if (out->history) {
     long long cap = out->history_rows;
     long long w = std::min(rows, cap);
@@ -2530,7 +2534,6 @@ extern "C" int apic_get_field(apic_sim* S, int32_t instance, int32_t which, doub
   if (!S || !out) return APIC_ERR_INVALID_ARG;
   if (instance < 0 || instance >= S->n_inst || which < 0 || which > 4) return APIC_ERR_INVALID_ARG;
   const Inst& I = S->inst[instance];
-  if (!S->sync()) return S->status;
   if (which == 0) S->d2h(out, S->d.rho + I.node_off, (size_t)I.nodes);
   else if (which == 1) S->d2h(out, S->d.phi + I.node_off, (size_t)I.nodes);
   else if (which == 4) S->d2h(out, S->d.V + I.node_off, (size_t)I.nodes);
