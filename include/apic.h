@@ -301,11 +301,12 @@ typedef struct {
                                     16384 nodes, up to 96 cells in x2) whose reduction blocks fit in L2 */
 #define APIC_SOLVER_ND 3         /* the same refinement around an FP32 nested-dissection factorisation (formed
                                     once at creation on the host in FP64) for some or all instances: the
-                                    default otherwise (larger grids, batches); APIC_DIRECT=bcr / nd / wide
-                                    (nested dissection only for grids wider than 256 cells) override */
-#define APIC_SOLVER_ND64 4       /* FP64 particles: the refinement around an FP64 nested-dissection factorisation
-                                    (one pass reaches FP64 rounding), the default; APIC_PRECOND=mg keeps
-                                    multigrid */
+                                    default otherwise (larger grids, batches); APIC_DIRECT=bcr / nd / nd64 /
+                                    wide (nested dissection only for grids wider than 256 cells) override */
+#define APIC_SOLVER_ND64 4       /* the refinement around an FP64 nested-dissection factorisation (one pass
+                                    reaches FP64 rounding): the default for FP64 particles (APIC_PRECOND=mg
+                                    keeps multigrid) and for one FP32 instance beyond the reduction's range of
+                                    up to 100000 nodes and 256 cells in x2 with a tolerance of 1e-9 or less */
 
 /* Counters of the batch (launch counts, Krylov iterations, phase times). */
 int apic_stats(apic_sim* sim, apic_stats_t* out);

@@ -1006,7 +1006,7 @@ static int setup(apic_sim* S) {
   NdUpload ndu;
   NdFlowPlan fp;       // the dataflow sweeps' records
   long long nd_w = 0;  // elements of one right-hand side's update vectors
-  constexpr int kElem = (int)(sizeof(Real) / sizeof(float));  // words per element of a dataflow solve's fronts
+  int elem = (int)(sizeof(Real) / sizeof(float));  // words per element of a dataflow solve's fronts
   {
     const char* pc = std::getenv("APIC_PRECOND");
     bool want = ni <= kCoopMaxInst && !(pc && std::string(pc) == "mg");
@@ -1014,12 +1014,22 @@ static int setup(apic_sim* S) {
     for (const Inst& I : S->inst) want = want && !(I.flags & (APIC_NO_FIELD | APIC_BOLTZMANN));
     const char* dm = std::getenv("APIC_DIRECT");
     const std::string direct = dm ? dm : "auto";
-    // auto: the reduction where every grid is small (its few phases are then
-    // shorter than the dissection's two sweeps over the tree) and all its
-    // blocks fit in L2, else the dissection (density, solve and fields, us:
-    // 64 x 32 61 and 91, 160 x 80 112 and 117, 192 x 96 138 and 124, 256 x 128
-    // 173 and 131, 96 x 200 188 and 122).  FP64 particles: the dissection (64 x
-    // 32 93 with multigrid's dense inverse and 66, 96 x 48 851 and 74)
+    // auto: FP64 fronts also for FP32 particles where one instance asks for a
+    // residual that takes FP32 fronts two passes (one leaves about 1e-7, so a
+    // tolerance of 1e-9 or less) and its grid is small: one pass of FP64 fronts
+    // is then shorter, the sweeps being bound by their chains of dependent
+    // fronts; on large ones and on batches the FP64 pipe and the bytes bound
+    // them (rows wider than 256 cells were not measured and keep FP32).
+    // The reduction where every grid is small (its few phases are then shorter
+    // than the dissection's two sweeps over the tree) and all its blocks fit
+    // in L2.  Density, solve and fields, us, reduction / FP32 / FP64 fronts:
+    // 64 x 32 61, 94, 72; 128 x 64 91, 116, 89; 160 x 80 114, 122, 103; 192 x
+    // 96 138, 124, -; 256 x 128 173, 136, 115; 96 x 200 170, 125, 104; 264 x
+    // 92 -, 132, 107; 512 x 256 -, 198, 193; 768 x 384 -, 274, 362; 1024 x 512
+    // -, 381, 568.  FP64 particles: the dissection (64 x 32 93 with
+    // multigrid's dense inverse and 66, 96 x 48 851 and 74)
+    const bool small64 = direct == "auto" && sizeof(Real) == 4 && ni == 1 && S->inst[0].tol <= 1e-9 &&
+                         S->inst[0].nodes <= 100000 && S->inst[0].N2 <= 257;
     bool red_fits = false;
     if (want && direct == "auto" && sizeof(Real) == 4) {
       double b = 0.0;
@@ -1031,11 +1041,12 @@ static int setup(apic_sim* S) {
       }
       red_fits = ok && b <= 112.0 * 1024 * 1024;
     }
+    if (direct == "nd64" || (small64 && !red_fits)) elem = 2;
     for (int k = 0; k < ni && want; ++k) {
       const Inst& I = S->inst[k];
       // wide: nested dissection only where the narrow reduction does not
       // apply (a batch may then mix both in one launch)
-      use_nd[k] = direct == "nd" || (direct == "auto" && !red_fits) || (direct == "wide" && I.N2 > kBcrMaxN + 1);
+      use_nd[k] = direct == "nd" || direct == "nd64" || (direct == "auto" && !red_fits) || (direct == "wide" && I.N2 > kBcrMaxN + 1);
       if (!use_nd[k]) continue;
       std::string why;
       int T = (int)std::min<unsigned>(16u, std::max(1u, std::thread::hardware_concurrency()));
@@ -1044,7 +1055,7 @@ static int setup(apic_sim* S) {
         const char* e = std::getenv("APIC_ND_LEAF");
         leaf = e ? std::max(1, std::min(256, std::atoi(e))) : 16;
       }
-      if (!nd_build(I.n1 - 1, I.N2, nd_coef, &levels[k][0], leaf, T, sizeof(Real) == 8, nds[k], why) ||
+      if (!nd_build(I.n1 - 1, I.N2, nd_coef, &levels[k][0], leaf, T, elem == 2, nds[k], why) ||
           nds[k].depth > kNdMaxDepth)
         use_nd[k] = 0;  // the reduction (or multigrid) instead
     }
@@ -1054,7 +1065,8 @@ static int setup(apic_sim* S) {
     bool flow = want;
     for (int k = 0; k < ni; ++k) flow = flow && use_nd[k];
     if (const char* e = std::getenv("APIC_ND_FLOW")) flow = flow && std::atoi(e) != 0;
-    if (flow) {
+    for (bool again = true; again && flow;) {
+      again = false;
       int dev = 0, sms = 0;
       cudaGetDevice(&dev);
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1075,12 +1087,13 @@ static int setup(apic_sim* S) {
         B.node_off = I.node_off;
         B.nodes = I.nodes;
         B.st_off = I.lv[0].st;
-        flow = nd_flow_add(fp, &nds[k], (int64_t)B.M * B.N, kElem, nd_workers(kElem) * ctas, nd_vec_cap(kElem),
-                           kElem == 1 ? kNdSum8Fronts * ctas : 1 << 30);
+        flow = nd_flow_add(fp, &nds[k], (int64_t)B.M * B.N, elem, nd_workers(elem) * ctas, nd_vec_cap(elem),
+                           elem == 1 ? kNdSum8Fronts * ctas : 1 << 30);
       }
       flow = flow && total_nodes < (1ll << 31);
       if (flow) {
-        pl.bcr.nd_elem = kElem;
+        pl.bcr.nd_elem = elem;
+        pl.bcr.nd_f64 = sizeof(Real) == 8;
         size_t fr = 0, tot = 0;
         if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) fr = 0;
         cudaGetLastError();
@@ -1098,6 +1111,10 @@ static int setup(apic_sim* S) {
       } else {  // a front beyond a record or a worker's vectors: level by level (FP32), multigrid (FP64)
         pl.bcr.nd_elem = 0;
         fp = NdFlowPlan();
+        if (sizeof(Real) == 4 && elem == 2) {  // (FP64 fronts hold the FP32 ones too)
+          elem = 1;
+          flow = again = true;
+        }
       }
     }
     if (sizeof(Real) == 8) want = want && flow;
@@ -1333,7 +1350,9 @@ static int setup(apic_sim* S) {
       S->h2d((int32_t*)d.nd_perm, fp.perm.data(), fp.perm.size());
       for (int k = 0; k < ni; ++k) {
         const NdFlowInst I{bcr_in[k].N, (int)bcr_in[k].foff, (int)bcr_in[k].node_off};
-        if (!upload_records<Real>(S, fp, k, I, nds[k], (int32_t*)d.bcr)) return S->status;
+        if (!(elem == 2 ? upload_records<double>(S, fp, k, I, nds[k], (int32_t*)d.bcr)
+                        : upload_records<float>(S, fp, k, I, nds[k], (int32_t*)d.bcr)))
+          return S->status;
         nds[k] = NdFactor();
       }
     } else if (!ndu.fronts.empty()) {

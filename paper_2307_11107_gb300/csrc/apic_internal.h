@@ -396,8 +396,9 @@ constexpr int kNdWarpMaxU = 192;    // ... and an update set up to this size
 #ifndef APIC_ND_UNITS
 #define APIC_ND_UNITS 4
 #endif
-// The dataflow sweeps split each solve CTA (16 warps) into kNdUnits workers,
-// each with its own task; the task limits follow from a worker's share.
+// Level by level (bcr.cu), each solve CTA of 16 warps takes kNdUnits tasks'
+// worth of limits: a task's rows, fronts and staged floats are a quarter of
+// the CTA's.
 constexpr int kNdUnits = APIC_ND_UNITS;
 constexpr int kNdWarpStage = 2048;    // matrix floats of a warp's front (staged in shared memory) at most
 constexpr int kNdStageFloats = 16 * kNdWarpStage;  // the CTA's stage
@@ -454,6 +455,7 @@ struct BcrPlan {
   int nd_floats;            // shared-memory floats a large nested-dissection front needs (0: none)
   int nd_elem;              // > 0: every instance by nested dissection, each sweep one dataflow phase (nd_solve.cu),
                             // in FP32 (1) or FP64 (2: words per matrix element)
+  int nd_f64;               // 1: FP64 particles
   int nd_nf, nd_nb;         // entries of the forward and backward record lists
   int nd_stream;            // 1: the records exceed L2 by far (copied with an evict-first hint)
 };

@@ -429,7 +429,7 @@ __device__ __forceinline__ void sweep(const DevPtrs& d, const BcrPlan& pl, const
 // mode, only, rhs as k_solve_bcr (bcr.cu).
 constexpr double kFloor64 = 1e-11;  // relative residual below which an FP64 solve may stop at its rounding floor
 
-template <class T>
+template <class T, class Real>  // of the fronts, of the particles
 __global__ void __launch_bounds__(nd_threads(sizeof(T) / 4), 1)
 k_solve_nd(const __grid_constant__ DevPtrs d, const __grid_constant__ BcrPlan pl, int mode, int only,
            const __grid_constant__ BcrRhs rhs) {
@@ -473,7 +473,7 @@ k_solve_nd(const __grid_constant__ DevPtrs d, const __grid_constant__ BcrPlan pl
     return r * r;
   };
   auto gradient = [&](const Inst& I, int nd) {
-    if constexpr (sizeof(T) == 4) grad_node<float, float2>(d, I, nd);
+    if constexpr (sizeof(Real) == 4) grad_node<float, float2>(d, I, nd);
     else grad_node<double, double2>(d, I, nd);
   };
   // the density and the first residual in one phase where every instance
@@ -615,7 +615,8 @@ k_nd_transposed(const __grid_constant__ DevPtrs d, const __grid_constant__ BcrPl
 }
 
 const void* kernel_of(const BcrPlan& b) {
-  return b.nd_elem == 2 ? (const void*)k_solve_nd<double> : (const void*)k_solve_nd<float>;
+  if (b.nd_elem == 1) return (const void*)k_solve_nd<float, float>;
+  return b.nd_f64 ? (const void*)k_solve_nd<double, double> : (const void*)k_solve_nd<double, float>;
 }
 
 }  // namespace
